@@ -64,8 +64,10 @@ enum {
 };
 
 enum {
-  AJF_PREC_F64 = 0,    /* FP64 arithmetic everywhere                                           */
-  AJF_PREC_F32 = 1,    /* GEMM-class steps on FP32 CUDA cores (operands rounded to FP32)       */
+  AJF_PREC_F64 = 0,    /* FP64 accuracy everywhere (GEMM-class steps: exact fp16 digit products
+                          on tcgen05, 64-bit fixed-point sums; FP64 CUDA cores without tcgen05) */
+  AJF_PREC_F32 = 1,    /* GEMM-class steps at FP32 accuracy (the same with fewer digits; FP32
+                          CUDA cores without tcgen05)                                          */
   AJF_PREC_TF32 = 2,   /* GEMM-class steps: one-pass TF32 tensor-core GEMMs (tcgen05), FP32 accumulate */
   AJF_PREC_TF32X3 = 3, /* split TF32 hi/lo operands, three tcgen05 products, FP32 accumulate   */
   AJF_PREC_BF16X3 = 4, /* bf16 operands split in two terms, three tcgen05 products             */
@@ -472,6 +474,17 @@ ajf_status ajf_selftest_queue_timeout(int device, double wait_ms, int32_t *code)
  * Errors: AJF_E_ARG, AJF_E_UNSUPPORTED (shape), AJF_E_NOMEM, AJF_E_CUDA, AJF_E_TIMEOUT. */
 ajf_status ajf_selftest_split_gemm(int device, int precision, int64_t M, int64_t N, int64_t K, const double *A,
                                    const double *B, double *C);
+
+/* Self-test of one complex product through the operand gather and the GEMM of the F64 (precision =
+ * AJF_PREC_F64) or F32 (AJF_PREC_F32) mode (no paper counterpart; used by the test suite):
+ * C[M][N] = A[M][K] . B[N][K]^T for complex128 A, B and C (interleaved, row-major, host memory), on
+ * device `device`. digits = 1: the fp16 digit product on the tensor cores; 0: the CUDA-core GEMM.
+ * order: bit order of the tensors that A and B are gathered from (0: k contiguous, 1: rows
+ * contiguous, 2: interleaved). M, N, K: powers of two with M >= 16, N >= 16, K >= 8. The call
+ * allocates and frees its own device memory and synchronises the device.
+ * Errors: AJF_E_ARG, AJF_E_UNSUPPORTED (shape), AJF_E_NOMEM, AJF_E_CUDA, AJF_E_TIMEOUT. */
+ajf_status ajf_selftest_digit_gemm(int device, int precision, int digits, int order, int64_t M, int64_t N, int64_t K,
+                                   const double *A, const double *B, double *C);
 
 /* Alg. I (alg = 1) or Alg. II (alg = 2) over several contexts at once: each context's device
  * program is enqueued on that context's own stream (give each context its own stream for the

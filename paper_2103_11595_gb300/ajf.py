@@ -133,6 +133,8 @@ def lib() -> ctypes.CDLL:
             "ajf_selftest_gemm": (I32, [ctypes.c_int, ctypes.c_int, ctypes.c_int, I64, I64, I64, P, P, P]),
             "ajf_fidelity_noalloc": (I32, [P, ctypes.c_int, D, ctypes.POINTER(Result)]),
             "ajf_selftest_split_gemm": (I32, [ctypes.c_int, ctypes.c_int, I64, I64, I64, P, P, P]),
+            "ajf_selftest_digit_gemm": (I32, [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, I64, I64, I64, P,
+                                              P, P]),
             "ajf_selftest_wait_timeout": (I32, [ctypes.c_int, D, ctypes.POINTER(I32)]),
             "ajf_learned_param_count": (I32, []),
             "ajf_set_learned_model": (I32, [P, P, I32]),
@@ -385,6 +387,22 @@ def ajf_selftest_split_gemm(device: int, precision: str, A: np.ndarray, B: np.nd
     st = lib().ajf_selftest_split_gemm(device, PRECISIONS[precision], M, N, K, _ptr(A), _ptr(B), _ptr(C))
     if st != AJF_OK:
         raise AjfError(st, "ajf_selftest_split_gemm failed")
+    return C
+
+
+def ajf_selftest_digit_gemm(device: int, precision: str, A: np.ndarray, B: np.ndarray, digits: bool = True,
+                            order: int = 0) -> np.ndarray:
+    """A @ B.T (complex128) through the gather and the GEMM of the "f64" or "f32" mode: fp16 digit
+    products on the tensor cores, or (digits=False) the CUDA-core GEMM."""
+    A = np.ascontiguousarray(A, dtype=np.complex128)
+    B = np.ascontiguousarray(B, dtype=np.complex128)
+    (M, K), (N, K2) = A.shape, B.shape
+    assert K == K2
+    C = np.empty((M, N), dtype=np.complex128)
+    st = lib().ajf_selftest_digit_gemm(device, PRECISIONS[precision], 1 if digits else 0, order, M, N, K, _ptr(A),
+                                       _ptr(B), _ptr(C))
+    if st != AJF_OK:
+        raise AjfError(st, "ajf_selftest_digit_gemm failed")
     return C
 
 

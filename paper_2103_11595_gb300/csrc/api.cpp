@@ -108,6 +108,10 @@ struct ajf_ctx {
   std::vector<int64_t> prog_key;
   bool prog_valid = false;
   int64_t prog_gen = 0;  // bumped whenever a new program is lowered
+  ajf::Program alt_prog;  // fixed-arena program of an F64 / F32 plan that outgrows that arena (plan_fixed_arena)
+  std::vector<char> alt_image;
+  int64_t alt_gen = -1;  // prog_gen it was made for
+  double plain_budget = 0;  // > 0: the program has CUDA-core GEMMs to meet this memory budget
   // tensor-core GEMM launches prepared on the host for (program, arena); index = launch index.
   // One set for the context's own arena, one for the fixed arena of ajf_fidelity_noalloc, so
   // that alternating the two paths re-encodes nothing.
@@ -423,7 +427,7 @@ ajf_status enqueue_program(ajf_ctx* c, cudaStream_t s, ajf_ctx::TcPrepSet* tc = 
   }
   for (size_t li = 0; li < P.launches.size(); ++li) {
     const Launch& ln = P.launches[li];
-    static const int kClass[6] = {1, 2, 3, 4, 5, 2};
+    static const int kClass[8] = {1, 2, 3, 4, 5, 2, 3, 5};
     ProfScope ps(c, s, kClass[ln.kind], ln.flops, ln.bytes);
     switch (ln.kind) {
       case LK_DOT:
@@ -445,6 +449,29 @@ ajf_status enqueue_program(ajf_ctx* c, cudaStream_t s, ajf_ctx::TcPrepSet* tc = 
       case LK_GEMM_TC:
         e = tc_gemm_run(tc->prep[li], s);
         break;
+      case LK_DIGITS:
+        e = cudaSuccess;
+        if (ln.row_exp) e = launch_row_exp(perms + ln.first, ln.count, ln.row_exp, ln.smem, arena, base, s);
+        if (e == cudaSuccess) e = launch_digits(perms + ln.first, ln.count, ln.blocks, ln.smem, arena, base, ln.mode, s);
+        break;
+      case LK_GEMM_DG: {
+        DgGemm g;
+        g.x = base + ln.a_off[0];
+        g.ex = reinterpret_cast<const int*>(base + ln.a_off[1]);
+        g.y = base + ln.b_off[0];
+        g.ey = reinterpret_cast<const int*>(base + ln.b_off[1]);
+        g.C = base + ln.c_off;
+        g.ws = reinterpret_cast<double*>(base + ln.ws_off);
+        g.status = reinterpret_cast<int*>(base + P.off_status);
+        g.M = ln.M;
+        g.N = ln.N;
+        g.K = ln.K;
+        g.ksplit = ln.ksplit;
+        g.mode = ln.mode;
+        g.wait_ns = kTcWaitNs;
+        e = launch_dg_gemm(g, s);
+        break;
+      }
       default:
         e = cudaErrorInvalidValue;
     }
@@ -852,7 +879,7 @@ ajf_status ajf_create(ajf_ctx** out, int device, void* cuda_stream) {
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return AJF_E_CUDA;
   c->tc_device = prop.major >= 10;
-  if (set_kernel_smem_limits() != cudaSuccess) return AJF_E_CUDA;
+  if (set_kernel_smem_limits() != cudaSuccess || set_dg_smem_limits() != cudaSuccess) return AJF_E_CUDA;
   // The fixed arena of ajf_fidelity_noalloc: its module is loaded (and the array reserved) here,
   // at set-up, so that the no-allocation call itself never triggers the reservation. Looked up
   // for every context, so a context created after a device reset sees the current address.
@@ -987,6 +1014,59 @@ ajf_status ajf_clear_noise(ajf_ctx* c) {
 
 namespace {
 
+// The descriptors of a program as they lie in the arena (leaves, steps, gathers, final pass).
+std::vector<char> descriptor_image(const Program& P) {
+  std::vector<char> img(P.desc_bytes, 0);
+  auto put = [&](size_t off, const void* src, size_t bytes) {
+    if (bytes) std::memcpy(img.data() + (off - P.off_desc), src, bytes);
+  };
+  put(P.off_leaves, P.leaves.data(), P.leaves.size() * sizeof(LeafDev));
+  put(P.off_steps, P.steps.data(), P.steps.size() * sizeof(StepDev));
+  put(P.off_perms, P.perms.data(), P.perms.size() * sizeof(PermDev));
+  put(P.off_final, &P.fin, sizeof(FinalDev));
+  return img;
+}
+
+// The planner's view of the options (no learned scorer).
+PlanParams plan_params(const ajf_plan_opts& o, bool tensor_cores) {
+  PlanParams pp;
+  pp.planner = o.planner;
+  pp.precision = o.precision;
+  pp.trials = o.trials;
+  pp.seed = o.seed;
+  pp.elem_bytes = o.precision == AJF_PREC_F64 ? 16 : 8;
+  pp.tensor_cores = tensor_cores;
+  switch (o.precision) {
+    case AJF_PREC_F64: pp.peak_flops = 1.0e12; break;
+    case AJF_PREC_F32: pp.peak_flops = 40e12; break;
+    case AJF_PREC_TF32: pp.peak_flops = 500e12; break;
+    case AJF_PREC_BF16X3: pp.peak_flops = 400e12; break;
+    default: pp.peak_flops = 200e12; break;
+  }
+  return pp;
+}
+
+// The program of the fixed arena (ajf_fidelity_noalloc): the context's own when it fits, else, for
+// the F64 and F32 modes (whose digit operands take more memory), one with CUDA-core GEMMs -- on the
+// same path, or on one planned for them. Kept until the next plan; `alt.prog.arena_bytes` is the
+// smallest found.
+void plan_fixed_arena(ajf_ctx* c) {
+  if (c->alt_gen == c->prog_gen) return;
+  auto consider = [&](const Path& path) {
+    Program p = lower(c->net, path, c->opts.precision, c->in.packed.size() / 2, c->tc_device, false, false);
+    if (c->alt_gen != c->prog_gen || p.arena_bytes < c->alt_prog.arena_bytes) c->alt_prog = std::move(p);
+    c->alt_gen = c->prog_gen;
+  };
+  consider(c->path);
+  if (c->alt_prog.arena_bytes > kStaticArenaBytes) {
+    PlanParams pp = plan_params(c->opts, false);
+    if (pp.planner == AJF_PLANNER_LEARNED) pp.planner = AJF_PLANNER_AUTO;
+    const Path path = plan_path(c->net, pp);
+    if (path.width <= kMaxBits - 2) consider(path);
+  }
+  c->alt_image = descriptor_image(c->alt_prog);
+}
+
 ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_info* info) {
   Range nvtx_range("ajf plan");
   if (!c) return AJF_E_ARG;
@@ -1079,7 +1159,12 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
   pkey.push_back(c->tc_device ? 1 : 0);
   pkey.push_back(o.slice_bonds);
   if (o.slice_bonds == AJF_SLICE_AUTO) pkey.push_back(static_cast<int64_t>(budget));
-  const bool prog_hit = c->prog_valid && pkey == c->prog_key;
+  // (a cached program with CUDA-core GEMMs in place of digit ones stands for budgets up to the one
+  // that asked for it, and one over this budget is lowered anew if that may make it fit)
+  const bool may_shrink = o.precision <= AJF_PREC_F32 && c->tc_device && o.lowering != AJF_LOWER_PERSISTENT;
+  const bool prog_hit = c->prog_valid && pkey == c->prog_key &&
+                        (c->plain_budget > 0 ? budget <= c->plain_budget
+                                             : !may_shrink || static_cast<double>(c->prog.arena_bytes) <= budget);
   bool cached = prog_hit;
   if (!prog_hit) {
     drop_graph(c);
@@ -1087,20 +1172,7 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
     cached = c->path_valid && key == c->plan_key;
     const Network full = (alg == 1) ? build_alg1(c->in, seq, sliced) : build_alg2(c->in, seq);
     c->net = full;
-    PlanParams pp;
-    pp.planner = o.planner;
-    pp.precision = o.precision;
-    pp.trials = o.trials;
-    pp.seed = o.seed;
-    pp.elem_bytes = o.precision == AJF_PREC_F64 ? 16 : 8;
-    pp.tensor_cores = c->tc_device;
-    switch (o.precision) {
-      case AJF_PREC_F64: pp.peak_flops = 1.0e12; break;
-      case AJF_PREC_F32: pp.peak_flops = 40e12; break;
-      case AJF_PREC_TF32: pp.peak_flops = 500e12; break;
-      case AJF_PREC_BF16X3: pp.peak_flops = 400e12; break;
-      default: pp.peak_flops = 200e12; break;
-    }
+    PlanParams pp = plan_params(o, c->tc_device);
     cudaError_t score_err = cudaSuccess;
     if (o.planner == AJF_PLANNER_LEARNED && static_cast<int>(c->mlp_weights.size()) == kMlpParams) {
       pp.mlp = c->mlp_weights.data();
@@ -1145,7 +1217,7 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
         }
       };
       bool lowered = false;
-      if (score_err == cudaSuccess) {
+      auto lower_path = [&](bool digits) {
         int count = o.slice_bonds > 0 ? o.slice_bonds : 0;
         if (o.slice_bonds == AJF_SLICE_AUTO) count = std::max(0, c->path_full.width - (kMaxBits - 2));
         for (;;) {
@@ -1153,11 +1225,27 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
           lowered = c->path.width <= kMaxBits - 2;
           if (lowered)
             c->prog = lower(c->net, c->path, o.precision, c->in.packed.size() / 2, c->tc_device,
-                            o.lowering == AJF_LOWER_PERSISTENT);
+                            o.lowering == AJF_LOWER_PERSISTENT, digits);
           if (o.slice_bonds != AJF_SLICE_AUTO) break;
           if (lowered && static_cast<double>(c->prog.arena_bytes) <= budget) break;
           if (count >= AJF_MAX_SLICE_BONDS || static_cast<int>(c->bond_labels.size()) < count) break;
           ++count;
+        }
+      };
+      if (score_err == cudaSuccess) lower_path(true);
+      // The digit operands of the F64 and F32 modes take up to 1.5 times the memory of the CUDA-core
+      // GEMMs', and the planner's model prefers wider paths with them. A plan over the budget is
+      // tried again with CUDA-core GEMMs, on the same path and then on one planned for them.
+      auto over = [&] { return !lowered || static_cast<double>(c->prog.arena_bytes) > budget; };
+      c->plain_budget = 0;
+      if (score_err == cudaSuccess && may_shrink && over()) {
+        c->plain_budget = budget;
+        lower_path(false);
+        if (over()) {
+          c->path_valid = false;  // the path below belongs to this budget only
+          pp.tensor_cores = false;
+          c->path_full = plan_path(full, pp);
+          if (score_err == cudaSuccess) lower_path(false);
         }
       }
       c->bond_leaves.clear();
@@ -1200,16 +1288,8 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
     c->prog_gen++;
   }
   const double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-  // descriptor image
   const Program& P = c->prog;
-  c->desc_image.assign(P.desc_bytes, 0);
-  if (!P.leaves.empty())
-    std::memcpy(c->desc_image.data() + (P.off_leaves - P.off_desc), P.leaves.data(), P.leaves.size() * sizeof(LeafDev));
-  if (!P.steps.empty())
-    std::memcpy(c->desc_image.data() + (P.off_steps - P.off_desc), P.steps.data(), P.steps.size() * sizeof(StepDev));
-  if (!P.perms.empty())
-    std::memcpy(c->desc_image.data() + (P.off_perms - P.off_desc), P.perms.data(), P.perms.size() * sizeof(PermDev));
-  std::memcpy(c->desc_image.data() + (P.off_final - P.off_desc), &P.fin, sizeof(FinalDev));
+  c->desc_image = descriptor_image(P);
   ajf_plan_info pi{};
   const int nb = static_cast<int>(c->bond_labels.size());
   pi.cmacs = std::ldexp(c->path.cmacs, nb);
@@ -1228,7 +1308,8 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
   pi.planner_used = c->path.planner;
   pi.n_launches = 3;  // leaves + final pass + final sum
   for (auto& ln : P.launches)
-    pi.n_launches += (ln.kind == LK_SPLITK || ln.kind == LK_DOT || (ln.kind == LK_GEMM_TC && ln.ksplit > 1)) ? 2 : 1;
+    pi.n_launches += (ln.kind == LK_SPLITK || ln.kind == LK_DOT || ln.row_exp > 0 ||
+                      ((ln.kind == LK_GEMM_TC || ln.kind == LK_GEMM_DG) && ln.ksplit > 1)) ? 2 : 1;
   pi.n_tc_gemms = P.tensor_cores;
   pi.plan_cached = cached ? 1 : 0;
   pi.n_removed = seq.removed;
@@ -1417,7 +1498,7 @@ ajf_status ajf_selftest_check_plan(ajf_ctx* c, int mutation) {
         }
         for (int k = ln.first; k < ln.first + ln.count; ++k)
           overwritten = overwritten || (P.steps[k].scalar_slot < 0 && hits(P.steps[k].c, P.steps[k].pc));
-      } else if (ln.kind == LK_PERM) {
+      } else if (ln.kind == LK_PERM || ln.kind == LK_DIGITS) {
         for (int k = ln.first; k < ln.first + ln.count; ++k)
           if (P.perms[k].src == from && P.perms[k].plane == plane && !P.perms[k].src_f32) P.perms[k].src = to;
       } else {
@@ -1502,7 +1583,7 @@ ajf_status ajf_selftest_check_plan(ajf_ctx* c, int mutation) {
     case 8: {  // a GEMM whose K is twice its gathers' (it would read past their operand terms)
       Launch* g = nullptr;
       for (auto& ln : P.launches)
-        if (!g && (ln.kind == LK_GEMM_TC || ln.kind == LK_GEMM_SIMT)) g = &ln;
+        if (!g && (ln.kind == LK_GEMM_TC || ln.kind == LK_GEMM_SIMT || ln.kind == LK_GEMM_DG)) g = &ln;
       if (!g) return fail(c, AJF_E_ARG, "no GEMM launch");
       g->K *= 2;
       break;
@@ -1584,6 +1665,29 @@ ajf_status ajf_fidelity_noalloc(ajf_ctx* c, int alg, double eps, ajf_result* out
   if (c->device < 0) return fail(c, AJF_E_STATE, "host-only context (device -1) cannot run the contraction");
   if (eps > 1.0) return fail(c, AJF_E_ARG, "eps > 1");
   if (multi_run(c)) return fail(c, AJF_E_STATE, "a sliced plan runs through ajf_fidelity_alg1/2 / ajf_fidelity only");
+  // A plan of the F64 or F32 mode that only its digit operands bring over the fixed arena runs with
+  // CUDA-core GEMMs there.
+  struct AltScope {  // swaps the fixed-arena program in for the call
+    ajf_ctx* c = nullptr;
+    void swap() {
+      std::swap(c->prog, c->alt_prog);
+      std::swap(c->desc_image, c->alt_image);
+    }
+    ~AltScope() {
+      if (c) swap();
+    }
+  } alt;
+  if (c->prog.arena_bytes > kStaticArenaBytes && c->opts.precision <= AJF_PREC_F32 && c->prog.tensor_cores > 0) {
+    try {
+      plan_fixed_arena(c);
+    } catch (const std::exception& ex) {
+      return fail(c, AJF_E_NOMEM, std::string("planning for the fixed arena failed: ") + ex.what());
+    }
+    if (c->alt_prog.arena_bytes <= kStaticArenaBytes) {
+      alt.c = c;
+      alt.swap();
+    }
+  }
   const Program& P = c->prog;
   if (P.arena_bytes > kStaticArenaBytes)
     return fail(c, AJF_E_NOMEM, "plan needs " + std::to_string(P.arena_bytes) + " bytes of device memory; the fixed " +
@@ -1877,6 +1981,141 @@ ajf_status ajf_selftest_split_gemm(int device, int precision, int64_t M, int64_t
   return st;
 }
 
+ajf_status ajf_selftest_digit_gemm(int device, int precision, int digits, int order, int64_t M, int64_t N, int64_t K,
+                                   const double* A, const double* B, double* C) {
+  if (!A || !B || !C || order < 0 || order > 2) return AJF_E_ARG;
+  if (precision != AJF_PREC_F64 && precision != AJF_PREC_F32) return AJF_E_ARG;
+  auto log2i = [](int64_t x) {
+    int b = 0;
+    while ((int64_t(1) << b) < x) ++b;
+    return (int64_t(1) << b) == x ? b : -1;
+  };
+  const int mb = log2i(M), nb = log2i(N), kb = log2i(K);
+  if (mb < 4 || nb < 4 || kb < 3 || mb + kb > 26 || nb + kb > 26 || mb + nb > 26) return AJF_E_UNSUPPORTED;
+  const int64_t Mt = 2 * M, Kt = 2 * K;
+  if (digits && !dg_gemm_supported(Mt, N, Kt)) return AJF_E_UNSUPPORTED;
+  if (cudaSetDevice(device) != cudaSuccess) return AJF_E_CUDA;
+  const bool f64 = precision == AJF_PREC_F64;
+  const int mode = digits ? (f64 ? OPM_DIG6 : OPM_DIG4) : (f64 ? OPM_F64 : OPM_F32);
+  const size_t eb = f64 ? 8 : 4;
+  auto al = [](size_t x) { return (x + 255) / 256 * 256; };
+  size_t top = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = top;
+    top += al(bytes);
+    return at;
+  };
+  PermDev pd[2];
+  size_t src[2], dig[2], exps[2], part[2];
+  int grid = 1, row_exp = 0;
+  size_t smem = 0;
+  for (int side = 0; side < 2; ++side) {
+    PermDev& q = pd[side];
+    std::memset(&q, 0, sizeof(q));
+    const int rb = side == 0 ? mb : nb;
+    q.rbits = rb;
+    q.kbits = kb;
+    q.plane = int64_t(1) << (rb + kb);
+    q.embed = side == 0 ? 1 : 0;
+    q.mode = mode;
+    q.rows.nbits = rb;
+    q.cols.nbits = kb;
+    // order 0: k bits lowest in the source, 1: row bits lowest, 2: interleaved
+    int r = 0, k = 0;
+    for (int pos = 0; pos < rb + kb; ++pos) {
+      const bool row = order == 0 ? k == kb : (order == 1 ? r < rb : (k == kb || (r < rb && (pos & 1))));
+      if (row) q.rows.pos[r++] = static_cast<int8_t>(pos);
+      else q.cols.pos[k++] = static_cast<int8_t>(pos);
+    }
+    q.rows_fast = q.rows.pos[0] == 0 ? 1 : 0;
+    src[side] = take(2 * size_t(q.plane) * 8);
+    q.src = static_cast<int64_t>(src[side] / 8);
+    const int64_t rows = side == 0 ? Mt : N;
+    if (digits) {
+      set_digit_tile(q);
+      dig[side] = take(dg_operand_bytes(rows, Kt, mode));
+      exps[side] = take((size_t(1) << rb) * 4);
+      part[side] = take((size_t(1) << rb) * 4 * static_cast<size_t>(std::max(1, q.strips)));
+      grid = static_cast<int>(std::max<int64_t>(grid, std::min<int64_t>(q.plane >> (q.tr + q.tk), 456)));
+      if (q.strips) row_exp = static_cast<int>(std::max<int64_t>(row_exp, std::min<int64_t>((int64_t(1) << (rb - q.tr)) * q.strips, 608)));
+    } else {
+      dig[side] = take(size_t(rows) * Kt * eb);
+      exps[side] = part[side] = 0;
+      grid = static_cast<int>(std::max<int64_t>(grid, std::min<int64_t>(std::max<int64_t>(q.plane >> 10, 1), 608)));
+    }
+    q.dst[0] = static_cast<int64_t>(dig[side]);
+    q.dst[1] = static_cast<int64_t>(exps[side]);
+    q.dst[2] = static_cast<int64_t>(part[side]);
+    smem = std::max(smem, perm_table_bytes(q));
+  }
+  const size_t c_off = take(size_t(Mt) * N * eb);
+  const int ksplit = digits ? dg_gemm_splits(Mt, N, Kt) : 1;
+  const size_t w_off = take(ksplit > 1 ? size_t(ksplit) * Mt * N * 8 : 8);
+  const size_t s_off = take(256), p_off = take(2 * sizeof(PermDev));
+  char* d = nullptr;
+  if (cudaMalloc(&d, top) != cudaSuccess) return AJF_E_NOMEM;
+  ajf_status st = AJF_OK;
+  std::vector<double> planar;
+  for (int side = 0; side < 2 && st == AJF_OK; ++side) {
+    const PermDev& q = pd[side];
+    const double* in = side == 0 ? A : B;
+    planar.assign(2 * size_t(q.plane), 0.0);
+    for (int64_t r = 0; r < (int64_t(1) << q.rbits); ++r)
+      for (int64_t k = 0; k < K; ++k) {
+        int64_t at = 0;
+        for (int i = 0; i < q.rbits; ++i) at += ((r >> i) & 1) << q.rows.pos[i];
+        for (int i = 0; i < kb; ++i) at += ((k >> i) & 1) << q.cols.pos[i];
+        planar[at] = in[2 * (r * K + k)];
+        planar[q.plane + at] = in[2 * (r * K + k) + 1];
+      }
+    if (cudaMemcpy(d + src[side], planar.data(), planar.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess) st = AJF_E_CUDA;
+  }
+  if (st == AJF_OK && (cudaMemcpy(d + p_off, pd, sizeof(pd), cudaMemcpyHostToDevice) != cudaSuccess ||
+                       cudaMemset(d + s_off, 0, 256) != cudaSuccess))
+    st = AJF_E_CUDA;
+  const PermDev* dp = reinterpret_cast<const PermDev*>(d + p_off);
+  cudaError_t e = cudaSuccess;
+  if (st == AJF_OK && digits) {
+    if (row_exp) e = launch_row_exp(dp, 2, row_exp, smem, d, d, 0);
+    if (e == cudaSuccess) e = launch_digits(dp, 2, grid, smem, d, d, mode, 0);
+    DgGemm g;
+    g.x = d + dig[0];
+    g.ex = reinterpret_cast<const int*>(d + exps[0]);
+    g.y = d + dig[1];
+    g.ey = reinterpret_cast<const int*>(d + exps[1]);
+    g.C = d + c_off;
+    g.ws = reinterpret_cast<double*>(d + w_off);
+    g.status = reinterpret_cast<int*>(d + s_off);
+    g.M = Mt;
+    g.N = N;
+    g.K = Kt;
+    g.ksplit = ksplit;
+    g.mode = mode;
+    g.wait_ns = kTcWaitNs;
+    if (e == cudaSuccess) e = launch_dg_gemm(g, 0);
+  } else if (st == AJF_OK) {
+    e = launch_perm(dp, 2, grid, smem, d, d, f64, 0);
+    if (e == cudaSuccess) e = launch_gemm_simt(d + dig[0], d + dig[1], d + c_off, Mt, N, Kt, f64, 0);
+  }
+  if (e != cudaSuccess) st = AJF_E_CUDA;
+  if (st == AJF_OK && cudaDeviceSynchronize() != cudaSuccess) st = AJF_E_CUDA;
+  int status = 0;
+  std::vector<char> cf(size_t(Mt) * N * eb);
+  if (st == AJF_OK && (cudaMemcpy(cf.data(), d + c_off, cf.size(), cudaMemcpyDeviceToHost) != cudaSuccess ||
+                       cudaMemcpy(&status, d + s_off, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess))
+    st = AJF_E_CUDA;
+  if (st == AJF_OK)
+    for (int64_t i = 0; i < M * N; ++i)
+      for (int pl = 0; pl < 2; ++pl) {
+        const size_t at = static_cast<size_t>(pl * M * N + i);
+        C[2 * i + pl] = f64 ? reinterpret_cast<const double*>(cf.data())[at]
+                            : static_cast<double>(reinterpret_cast<const float*>(cf.data())[at]);
+      }
+  if (st == AJF_OK && status != 0) st = AJF_E_TIMEOUT;
+  cudaFree(d);
+  return st;
+}
+
 ajf_status ajf_plan_launches(const ajf_ctx* c, ajf_launch_info* out, int cap, int* n) {
   if (!c || !n || cap < 0 || (cap > 0 && !out)) return AJF_E_ARG;
   if (!c->planned) return AJF_E_STATE;
@@ -1893,9 +2132,10 @@ ajf_status ajf_plan_launches(const ajf_ctx* c, ajf_launch_info* out, int cap, in
     v.push_back(li);
   };
   add(0, 0, 0, 0, 0, 0, 0);
-  static const int kClass[6] = {1, 2, 3, 4, 5, 2};
+  static const int kClass[8] = {1, 2, 3, 4, 5, 2, 3, 5};
   for (const Launch& ln : c->prog.launches) {
-    add(kClass[ln.kind], ln.kind == LK_GEMM_TC ? ln.npass : (ln.kind == LK_GEMM_SIMT ? 1 : 0), ln.M, ln.N, ln.K,
+    add(kClass[ln.kind], ln.kind == LK_GEMM_TC || ln.kind == LK_GEMM_DG ? ln.npass : (ln.kind == LK_GEMM_SIMT ? 1 : 0),
+        ln.M, ln.N, ln.K,
         ln.flops, ln.bytes);
     if (ln.kind == LK_SPLITK || ln.kind == LK_DOT) add(2, 0, 0, 0, 0, 0, 0);  // the deterministic final-sum launch
   }
@@ -2384,6 +2624,8 @@ ajf_status queue_table(ajf_ctx* const* ctxs, int n, double* dev_results, const Q
           ph.desc = perms + ln.first;
           add(ph, -1);
           break;
+        case LK_DIGITS:
+          return fail(c, AJF_E_UNSUPPORTED, "step interpreter: FP64 or FP32 GEMM operands (use a tensor-core mode)");
         case LK_GEMM_TC: {
           int bn = 0, bf16 = 0, nwork = 0;
           const size_t at = params.size();

@@ -8,6 +8,8 @@
 // where bit i is the tensor's i-th label. Scalars produced by full contractions are FP64 (double2
 // slots).
 #pragma once
+#include <cuda_runtime.h>
+
 #include <cstdint>
 
 namespace ajf {
@@ -54,6 +56,14 @@ struct PermDev {
   int32_t rows_fast;      // 1: read with lanes along rows (the source's stride-1 bit is a row bit)
   int32_t mode;           // operand format, see OperandMode
   int32_t src_f32;        // the source is complex64 (FP32 planes), else complex128
+  // digit operands only (OPM_DIG6, OPM_DIG4; digits.cuh): dst[0] is the digit array, dst[1] the
+  // row exponents (int32 exponent field per complex row), dst[2] per-strip exponents when K is
+  // longer than a tile. A tile is 2^tr rows x 2^tk k; its bits are listed by source position
+  // (element l of the tile: bit j of l adds 2^tsrc[j] to the source offset and is bit tloc[j] of
+  // row * 2^tk + k), so that consecutive l are as contiguous in the source as the tile allows.
+  int32_t tr, tk;
+  int32_t strips;         // strips of the row-exponent pass (0: K fits a tile, no pass)
+  int8_t tsrc[12], tloc[12];
 };
 
 enum OperandMode : int32_t {
@@ -65,7 +75,11 @@ enum OperandMode : int32_t {
   OPM_BF16X3 = 5,  // hi, mid, lo (bf16)
   OPM_F16X2S = 6,  // hi, lo (fp16) of x / q, with q a power of two per row and K block (dst[2]: the
                    // FP32 q's, [K block][row])
+  OPM_DIG6 = 7,    // six fixed-point fp16 digits of a row-wise quantum (FP64 GEMMs)
+  OPM_DIG4 = 8,    // four digits (GEMMs of the FP32 mode)
 };
+
+__host__ __device__ constexpr bool digit_mode(int mode) { return mode == OPM_DIG6 || mode == OPM_DIG4; }
 
 // Leaf construction from the uploaded complex128 inputs.
 struct LeafDev {

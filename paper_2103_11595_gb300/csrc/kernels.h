@@ -41,6 +41,32 @@ cudaError_t launch_persistent(const InterpJob* d_jobs, int n_jobs, const InterpO
                               cudaStream_t s);
 constexpr size_t kPersistentSmemMax = 96 * 1024;
 
+// GEMMs of the FP64 and FP32 modes on the fp16 tensor cores (dg_gemm.cu, digits.cuh): bytes of a
+// digit operand (rows x kcols real columns), supported shapes and K splits.
+size_t dg_operand_bytes(int64_t rows, int64_t kcols, int mode);
+bool dg_gemm_supported(int64_t M, int64_t N, int64_t K);
+int dg_gemm_splits(int64_t M, int64_t N, int64_t K);
+// Row exponents of the operands whose K spans several gather tiles (PermDev::strips > 0), then the
+// gather itself; `mode` is the (common) digit mode of the perms.
+cudaError_t launch_row_exp(const PermDev* d_perms, int nperm, int grid_x, size_t smem, const void* arena, void* base,
+                           cudaStream_t s);
+cudaError_t launch_digits(const PermDev* d_perms, int nperm, int grid_x, size_t smem, const void* arena, void* base,
+                          int mode, cudaStream_t s);
+struct DgGemm {
+  const void* x = nullptr;   // X digits (M rows: embedded complex rows), Y digits (N rows)
+  const void* y = nullptr;
+  const int* ex = nullptr;   // row exponent fields: M / 2 and N values
+  const int* ey = nullptr;
+  void* C = nullptr;         // M x N, FP64 (OPM_DIG6) or FP32 (OPM_DIG4)
+  double* ws = nullptr;      // ksplit > 1: ksplit * M * N FP64 partials
+  int* status = nullptr;
+  int64_t M = 0, N = 0, K = 0;
+  int ksplit = 1, mode = OPM_DIG6;
+  unsigned long long wait_ns = 0;  // bound of every device-side wait
+};
+cudaError_t launch_dg_gemm(const DgGemm& g, cudaStream_t s);
+cudaError_t set_dg_smem_limits();
+
 // Tensor-core GEMM (tcgen05, tc_gemm.cu): C[M][N] (FP32, row-major) =
 // sum_{i + j < terms} A_i[M][K] . B_j[N][K]^T for the split terms A_t, B_t (byte offsets from
 // `base`), FP32 accumulation promoted per K block. kind 0: tf32, 1: bf16, 2: scaled fp16.

@@ -129,7 +129,16 @@ double step_seconds(int ra, int rb, int runion, int rc, const PlanParams& p) {
   const bool tc = p.tensor_cores && p.precision >= AJF_PREC_TF32;
   int terms = 1, passes = 1;
   double eb = 8, rate = kFp64, tm = 64, tn = 64;
-  if (p.precision == AJF_PREC_F32) {
+  if (p.tensor_cores && !tc) {
+    // F64, F32: fp16 digit products (dg_gemm.cu)
+    const bool f64 = p.precision == AJF_PREC_F64;
+    terms = f64 ? 6 : 4;
+    passes = f64 ? 26 : 10;
+    eb = 2;
+    rate = 1.1e15;
+    tm = Mt >= 128 ? 128 : Mt;
+    tn = 128;
+  } else if (p.precision == AJF_PREC_F32) {
     eb = 4;
     rate = kFp32;
     tm = 128;
@@ -146,7 +155,7 @@ double step_seconds(int ra, int rb, int runion, int rc, const PlanParams& p) {
   const double gather = (std::ldexp(1.0, ra) + std::ldexp(1.0, rb)) * p.elem_bytes + operands;
   const double out = Mt * Nt * p.elem_bytes / 2;  // real planes of the complex result
   double tiles = std::ceil(Mt / tm) * std::ceil(Nt / tn);
-  if (tc) tiles *= std::max(1.0, std::min(std::ceil(kSMs / tiles) * 2.0, Kt * eb / 1024.0));  // K splits
+  if (p.tensor_cores) tiles *= std::max(1.0, std::min(std::ceil(kSMs / tiles) * 2.0, Kt * eb / 1024.0));  // K splits
   const double eff = std::min(1.0, tiles / kSMs);
   return gather / kGatherBw + std::max(passes * flops / (rate * eff), (operands + out) / kBw) + 14e-6;
 }

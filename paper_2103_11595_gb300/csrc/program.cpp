@@ -5,8 +5,9 @@
 //   GEMM   -- M, N >= 16, K >= 8 and M*N*K >= 2^18: both operands are gathered into real,
 //             K-contiguous GEMM operands (the smaller one embedded as [[Re,-Im],[Im,Re]]) and one
 //             real GEMM C' = X' Y'^T produces C directly in planar layout with labels
-//             (n-bits low, m-bits high). GEMMs run on tcgen05 in the tensor-core precision modes
-//             when the shape is tile-aligned, else on CUDA cores.
+//             (n-bits low, m-bits high). GEMMs run on tcgen05: in the tensor-core precision modes
+//             on split operands, in the F64 and F32 modes as digit products (dg_gemm.cu); on CUDA
+//             cores where there is no tcgen05 or the memory budget has no room for the digits.
 //   SPLITK -- full contractions to a scalar (the trace) and steps with <= 2^12 outputs and a
 //             contracted index of >= 2^10: FP64 partial sums, deterministic final sum.
 //   SMALL  -- everything else (gate absorption, outer products, tiny merges): one thread per
@@ -123,8 +124,26 @@ size_t mode_bytes(int mode) { return mode == OPM_F64 ? 8 : (mode >= OPM_BF16X2 ?
 
 }  // namespace
 
+void set_digit_tile(PermDev& d) {
+  // up to 64 k (one 64-column chunk of a plane) x as many rows as make 2048 elements, its bits
+  // listed by source position
+  d.tk = std::min(d.kbits, 6);
+  d.tr = std::min(d.rbits, 11 - d.tk);
+  std::vector<std::pair<int, int>> bits;  // (source position, local bit)
+  for (int q = 0; q < d.tk; ++q) bits.emplace_back(d.cols.pos[q], q);
+  for (int q = 0; q < d.tr; ++q) bits.emplace_back(d.rows.pos[q], d.tk + q);
+  std::sort(bits.begin(), bits.end());
+  for (size_t q = 0; q < bits.size(); ++q) {
+    d.tsrc[q] = static_cast<int8_t>(bits[q].first);
+    d.tloc[q] = static_cast<int8_t>(bits[q].second);
+  }
+  // rows longer than a tile: their exponents come from a pass of their own, over up to 16 strips
+  // of K per row tile
+  d.strips = d.kbits > d.tk ? std::min(1 << (d.kbits - d.tk), 16) : 0;
+}
+
 Program lower(const Network& net, const Path& path, int precision, size_t inputs_complex, bool tc_ok,
-              bool persistent) {
+              bool persistent, bool digits) {
   Program P;
   P.persistent = persistent;
   P.alg = net.alg;
@@ -266,6 +285,95 @@ Program lower(const Network& net, const Path& path, int precision, size_t inputs
   };
   std::vector<int> gemm_launches;
 
+  // GEMM-class step `s` of the F64 and F32 modes on the fp16 tensor cores: digit gathers and the
+  // digit product (dg_gemm.cu). xf, yf: the free labels of the operands.
+  auto lower_digits = [&](int s, const std::vector<int>& xf, const std::vector<int>& yf) {
+    const StepInfo& I = info[s];
+    const int c = L + s;
+    const int64_t Mt = int64_t(1) << (I.m + 1), Nt = int64_t(1) << I.n, Kt = int64_t(1) << (I.k + 1);
+    const bool f64 = precision == AJF_PREC_F64;
+    const int dmode = f64 ? OPM_DIG6 : OPM_DIG4;
+    PermDev pd[2];
+    size_t dig[2], exps[2], part[2], dig_bytes[2], exp_bytes[2], part_bytes[2];
+    Launch lp;
+    lp.kind = LK_DIGITS;
+    lp.mode = dmode;
+    lp.op_f64 = f64 ? 1 : 0;
+    lp.first = static_cast<int>(P.perms.size());
+    lp.count = 2;
+    int64_t tiles = 1, strip_items = 0;
+    for (int side = 0; side < 2; ++side) {
+      const int id = side == 0 ? I.a : I.b;
+      const auto& lab = labels[id];
+      const auto& rows = side == 0 ? xf : yf;
+      PermDev& d = pd[side];
+      std::memset(&d, 0, sizeof(d));
+      d.src = static_cast<int64_t>(toff[id] / elem(id));
+      d.src_f32 = t32[id];
+      d.plane = int64_t(1) << lab.size();
+      d.rows = make_map(rows, lab);
+      d.cols = make_map(I.shared, lab);
+      d.rbits = static_cast<int32_t>(rows.size());
+      d.kbits = I.k;
+      d.embed = side == 0 ? 1 : 0;
+      d.mode = dmode;
+      set_digit_tile(d);
+      dig_bytes[side] = dg_operand_bytes(side == 0 ? Mt : Nt, Kt, dmode);
+      exp_bytes[side] = (size_t(1) << d.rbits) * 4;
+      part_bytes[side] = exp_bytes[side] * static_cast<size_t>(d.strips);
+      dig[side] = ff.alloc(dig_bytes[side]);
+      exps[side] = ff.alloc(exp_bytes[side]);
+      part[side] = d.strips ? ff.alloc(part_bytes[side]) : 0;
+      d.dst[0] = static_cast<int64_t>(dig[side]);
+      d.dst[1] = static_cast<int64_t>(exps[side]);
+      d.dst[2] = static_cast<int64_t>(part[side]);
+      tiles = std::max(tiles, int64_t(1) << (d.rbits + d.kbits - d.tr - d.tk));
+      if (d.strips) strip_items = std::max(strip_items, (int64_t(1) << (d.rbits - d.tr)) * d.strips);
+      lp.smem = std::max(lp.smem, perm_table_bytes(d));
+      lp.bytes += std::ldexp(1.0, static_cast<int>(lab.size())) * elem(id) * 2.0 + static_cast<double>(dig_bytes[side]);
+      P.perms.push_back(d);
+    }
+    // at most four (row exponents) or three (gather) resident blocks per SM, several tiles each
+    lp.blocks = static_cast<int>(std::min<int64_t>(tiles, 3 * 152));
+    lp.row_exp = static_cast<int>(std::min<int64_t>(strip_items, 4 * 152));
+    P.launches.push_back(lp);
+    release_dead(exec_pos[s], {I.a, I.b});
+    for (int side = 0; side < 2; ++side)
+      if (part_bytes[side]) ff.release(part[side], part_bytes[side]);
+    t32[c] = f64 ? 0 : 1;
+    toff[c] = ff.alloc(tensor_bytes(c));
+    const int ksplit = dg_gemm_splits(Mt, Nt, Kt);
+    const size_t ws_bytes = ksplit > 1 ? size_t(ksplit) * size_t(Mt) * size_t(Nt) * 8 : 0;  // FP64 partials
+    const size_t ws = ws_bytes ? ff.alloc(ws_bytes) : 0;
+    Launch lg;
+    lg.kind = LK_GEMM_DG;
+    lg.mode = dmode;
+    lg.op_f64 = f64 ? 1 : 0;
+    lg.npass = f64 ? 6 : 4;
+    lg.ksplit = ksplit;
+    lg.ws_off = static_cast<int64_t>(ws);
+    lg.M = Mt;
+    lg.N = Nt;
+    lg.K = Kt;
+    lg.a_off[0] = static_cast<int64_t>(dig[0]);
+    lg.a_off[1] = static_cast<int64_t>(exps[0]);
+    lg.b_off[0] = static_cast<int64_t>(dig[1]);
+    lg.b_off[1] = static_cast<int64_t>(exps[1]);
+    lg.c_off = static_cast<int64_t>(toff[c]);
+    lg.flops = 8.0 * std::ldexp(1.0, I.m + I.n + I.k);
+    lg.bytes = (std::ldexp(1.0, static_cast<int>(labels[I.a].size())) * elem(I.a) +
+                std::ldexp(1.0, static_cast<int>(labels[I.b].size())) * elem(I.b) +
+                std::ldexp(1.0, static_cast<int>(labels[c].size())) * elem(c)) * 2.0;
+    gemm_launches.push_back(static_cast<int>(P.launches.size()));
+    P.launches.push_back(lg);
+    P.tensor_cores++;
+    for (int side = 0; side < 2; ++side) {
+      ff.release(dig[side], dig_bytes[side]);
+      ff.release(exps[side], exp_bytes[side]);
+    }
+    if (ws_bytes) ff.release(ws, ws_bytes);
+  };
+
   int i = 0;
   while (i < S) {
     const int s0 = order[i];
@@ -381,6 +489,11 @@ Program lower(const Network& net, const Path& path, int precision, size_t inputs
       for (int v : ly)
         if (!contains(I.shared, v)) yf.push_back(v);
       const int64_t Mt = int64_t(1) << (I.m + 1), Nt = int64_t(1) << I.n, Kt = int64_t(1) << (I.k + 1);
+      if (tc_ok && digits && precision <= AJF_PREC_F32 && dg_gemm_supported(Mt, Nt, Kt)) {
+        lower_digits(s, xf, yf);
+        ++i;
+        continue;
+      }
       const bool use_tc = tc_ok && precision >= AJF_PREC_TF32 && tc_gemm_supported(Mt, Nt, Kt, tc_kind);
       const bool op_f64 = !use_tc && precision == AJF_PREC_F64;
       const int gmode = use_tc ? mode : (op_f64 ? OPM_F64 : OPM_F32);
@@ -769,6 +882,69 @@ std::string check_program(const Program& P) {
           if (!in_work(d)) return ws + ": scale array outside the work region";
           W.push_back(d);
         }
+      }
+    } else if (ln.kind == LK_DIGITS) {
+      if (ln.count != 2 || ln.first < 0 || ln.first + 2 > static_cast<int>(P.perms.size())) return who + ": gather range";
+      for (int k = ln.first; k < ln.first + 2; ++k) {
+        const PermDev& g = P.perms[k];
+        const std::string ws = who + " gather " + std::to_string(k);
+        const int bp = log2_exact(g.plane);
+        if (bp < 0 || g.rows.nbits != g.rbits || g.cols.nbits != g.kbits) return ws + ": map sizes";
+        uint64_t used = 0;
+        if (!add_positions(g.rows, bp, used) || !add_positions(g.cols, bp, used))
+          return ws + ": source addresses repeat or overflow";
+        if (used != (uint64_t(1) << bp) - 1) return ws + ": a source bit is not addressed";
+        // the tile's bits: each local bit once, at the source position of its row or k bit
+        if (g.tk < 3 || g.tk > 6 || g.tk > g.kbits || g.tr < 0 || g.tr > g.rbits || g.tr + g.tk > 11 || g.mode != ln.mode ||
+            !digit_mode(g.mode))
+          return ws + ": gather tile";
+        uint32_t seen = 0;
+        for (int q = 0; q < g.tr + g.tk; ++q) {
+          const int b = g.tloc[q];
+          if (b < 0 || b >= g.tr + g.tk || ((seen >> b) & 1)) return ws + ": gather tile bits";
+          seen |= 1u << b;
+          if (g.tsrc[q] != (b < g.tk ? g.cols.pos[b] : g.rows.pos[b - g.tk])) return ws + ": gather tile positions";
+        }
+        const int64_t nkt = int64_t(1) << (g.kbits - g.tk);
+        if (nkt == 1 ? g.strips != 0 : (g.strips < 1 || nkt % g.strips != 0 || ln.row_exp < 1)) return ws + ": row strips";
+        const Span src = tensor(g.src, g.plane, g.src_f32);
+        if (!in_work(src)) return ws + ": source outside the work region";
+        R.push_back(src);
+        const size_t rows = size_t(1) << g.rbits;
+        const size_t db = dg_operand_bytes(static_cast<int64_t>(rows) << (g.embed ? 1 : 0), int64_t(2) << g.kbits, g.mode);
+        const size_t sizes[3] = {db, rows * 4, rows * 4 * static_cast<size_t>(g.strips)};
+        for (int t = 0; t < (g.strips ? 3 : 2); ++t) {
+          const Span d{static_cast<size_t>(g.dst[t]), static_cast<size_t>(g.dst[t]) + sizes[t]};
+          if (!in_work(d)) return ws + ": operand array " + std::to_string(t) + " outside the work region";
+          W.push_back(d);
+        }
+      }
+    } else if (ln.kind == LK_GEMM_DG) {
+      if (li == 0 || P.launches[li - 1].kind != LK_DIGITS) return who + ": GEMM without its gather";
+      const Launch& lp = P.launches[li - 1];
+      const PermDev& px = P.perms[lp.first];
+      const PermDev& py = P.perms[lp.first + 1];
+      if (px.embed != 1 || py.embed != 0 || px.kbits != py.kbits || px.mode != py.mode || px.mode != ln.mode ||
+          ln.M != (int64_t(2) << px.rbits) || ln.N != (int64_t(1) << py.rbits) || ln.K != (int64_t(2) << px.kbits))
+        return who + ": GEMM shape differs from its gathers";
+      if (!dg_gemm_supported(ln.M, ln.N, ln.K)) return who + ": GEMM shape";
+      const int64_t offs[4] = {ln.a_off[0], ln.a_off[1], ln.b_off[0], ln.b_off[1]};
+      const size_t sizes[4] = {dg_operand_bytes(ln.M, ln.K, ln.mode), size_t(ln.M / 2) * 4,
+                               dg_operand_bytes(ln.N, ln.K, ln.mode), size_t(ln.N) * 4};
+      for (int t = 0; t < 4; ++t) {
+        const Span d{static_cast<size_t>(offs[t]), static_cast<size_t>(offs[t]) + sizes[t]};
+        if (!in_work(d)) return who + ": operand outside the work region";
+        R.push_back(d);
+      }
+      const size_t ce = ln.mode == OPM_DIG6 ? 8 : 4;
+      const Span c{static_cast<size_t>(ln.c_off), static_cast<size_t>(ln.c_off) + size_t(ln.M) * size_t(ln.N) * ce};
+      if (!in_work(c)) return who + ": result outside the work region";
+      W.push_back(c);
+      if (ln.ksplit > 1) {
+        const Span w{static_cast<size_t>(ln.ws_off),
+                     static_cast<size_t>(ln.ws_off) + size_t(ln.ksplit) * size_t(ln.M) * size_t(ln.N) * 8};
+        if (!in_work(w)) return who + ": K-split workspace outside the work region";
+        W.push_back(w);
       }
     } else if (ln.kind == LK_GEMM_TC || ln.kind == LK_GEMM_SIMT) {
       if (li == 0 || P.launches[li - 1].kind != LK_PERM) return who + ": GEMM without its gather";

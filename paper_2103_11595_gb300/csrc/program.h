@@ -9,7 +9,8 @@
 
 namespace ajf {
 
-enum LaunchKind : int32_t { LK_SMALL = 0, LK_SPLITK = 1, LK_PERM = 2, LK_GEMM_SIMT = 3, LK_GEMM_TC = 4, LK_DOT = 5 };
+enum LaunchKind : int32_t { LK_SMALL = 0, LK_SPLITK = 1, LK_PERM = 2, LK_GEMM_SIMT = 3, LK_GEMM_TC = 4, LK_DOT = 5,
+                            LK_DIGITS = 6, LK_GEMM_DG = 7 };
 
 struct Launch {
   int32_t kind = 0;
@@ -19,11 +20,13 @@ struct Launch {
   // GEMM: C[M][N] = sum_p A_p[M][K] . B_p[N][K]^T (byte offsets into the arena)
   int64_t a_off[6] = {0, 0, 0, 0, 0, 0}, b_off[6] = {0, 0, 0, 0, 0, 0};
   int32_t npass = 0;
-  int32_t tc_kind = 0;           // 0 tf32, 1 bf16
+  int32_t tc_kind = 0;           // 0 tf32, 1 bf16, 2 scaled fp16
+  int32_t mode = 0;              // DIGITS, GEMM_DG: OperandMode (a_off / b_off: X / Y digits, row exponents)
   int32_t op_f64 = 1;            // CUDA-core GEMM: FP64 (1) or FP32 (0) operands
+  int32_t row_exp = 0;           // DIGITS: grid of the row-exponent pass that goes first (0: none)
   int64_t c_off = 0;             // byte offset of C
   int32_t ksplit = 1;            // tensor-core GEMM: K splits (> 1: FP32 partials in the workspace)
-  int64_t ws_off = 0;            // byte offset of the split workspace (ksplit * M * N floats)
+  int64_t ws_off = 0;            // byte offset of the split workspace (ksplit * M * N floats; doubles in GEMM_DG)
   int64_t M = 0, N = 0, K = 0;
   double flops = 0, bytes = 0;   // algorithmic work of the complex step this launch belongs to
 };
@@ -62,11 +65,16 @@ struct Program {
 };
 
 // Lower `path` over `net` to a device program for `precision`. `inputs_complex` is the number
-// of complex128 values in the packed input buffer. `tc_ok`: tensor-core GEMMs may be used.
+// of complex128 values in the packed input buffer. `tc_ok`: tensor-core GEMMs may be used;
+// `digits`: also those of the F64 and F32 modes (digit operands, which take up to 1.5 times the
+// memory of the CUDA-core GEMMs' operands).
 // `persistent`: every step becomes a CUDA-core gather step (LK_SMALL) or a reduction step
 // (LK_SPLITK), so that one thread block of the persistent kernel can run the whole program.
 Program lower(const Network& net, const Path& path, int precision, size_t inputs_complex, bool tc_ok,
-              bool persistent = false);
+              bool persistent = false, bool digits = true);
+
+// Gather tile and row-exponent strips of a digit operand (PermDev::tr .. tloc) from its maps.
+void set_digit_tile(PermDev& d);
 
 // Host-side replay of a lowered program's address arithmetic and buffer lifetimes (no device
 // needed): "" if every access stays inside its buffer and region and no launch overwrites a buffer

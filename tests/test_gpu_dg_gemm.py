@@ -1,0 +1,92 @@
+"""The fp16 digit products that carry the GEMM-class steps of the F64 and F32 modes, through the
+path's own gather and GEMM, against extended-precision products and the CUDA-core GEMMs."""
+import numpy as np
+import pytest
+
+from paper_2103_11595_gb300 import ajf, workloads as W
+
+# shapes (complex M, N, K): the smallest; 2 and 4 digits per 128-byte row (K = 16, 8); X tiles of 32,
+# 64 and 128 rows; Y tiles with and without missing rows; one and several K chunks and strips; K splits
+SHAPES = [(16, 16, 8), (16, 256, 16), (32, 128, 8), (64, 32, 32), (128, 256, 32), (16, 512, 64), (256, 16, 128),
+          (64, 64, 512), (16, 32, 4096)]
+
+
+def operands(M, N, K, dist, seed):
+    r = np.random.default_rng(seed)
+    A = r.standard_normal((M, K)) + 1j * r.standard_normal((M, K))
+    B = r.standard_normal((N, K)) + 1j * r.standard_normal((N, K))
+    if dist == "equal":  # every digit of every entry the same: the largest sums the tensor core can see
+        A = np.full((M, K), 1.9999999999999998 * (1 + 1j))
+        B = np.full((N, K), -1.9999999999999998 * (1 - 1j))
+    elif dist == "graded":
+        A = A * 10.0 ** r.uniform(-200, 0, (M, 1)) * 10.0 ** r.uniform(-3, 0, (M, K))
+        B = B * 10.0 ** r.uniform(-3, 0, (N, K))
+        A[1], B[2] = 0, 0
+    return A, B
+
+
+def exact(A, B):
+    a, b, c, d = (x.astype(np.longdouble) for x in (A.real, A.imag, B.real, B.imag))
+    return a @ c.T - b @ d.T, a @ d.T + b @ c.T
+
+
+def bound(A, B, R, f32):
+    """Element bound. Digits: 2^-56 (F64) or 2^-38 of the row maximum per factor, the dropped levels
+    less than that again, over 2K products; the fixed-point sum: up to three roundings per chunk of
+    64 columns in units of 2^-54 (chunks per sum) of the maxima's product; the result's own rounding."""
+    K2 = 2 * A.shape[1]
+    m = np.maximum(abs(A.real), abs(A.imag)).max(1)[:, None] * np.maximum(abs(B.real), abs(B.imag)).max(1)[None, :]
+    chunks = max(1, K2 // 64)
+    c = min(chunks, 32)
+    per = K2 * 4 * (2.0 ** -38 if f32 else 2.0 ** -56) + 1.5 * chunks * c * 2.0 ** -54
+    return 2.0 ** (-24 if f32 else -53) * 1.01 * np.maximum(abs(R[0]), abs(R[1])).astype(float) + m * per
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_digit_gemm_against_extended_precision(precision, shape):
+    for dist in ("normal", "equal", "graded"):
+        if precision == "f32" and dist == "graded":
+            continue  # FP32 results would leave their range
+        A, B = operands(*shape, dist, 7)
+        R = exact(A, B)
+        got = [ajf.ajf_selftest_digit_gemm(0, precision, A, B, order=o) for o in (0, 1, 2)]
+        assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])  # any source bit order
+        err = np.maximum(abs(got[0].real - R[0]), abs(got[0].imag - R[1])).astype(float)
+        assert (err <= bound(A, B, R, precision == "f32")).all(), (dist, (err / bound(A, B, R, precision == "f32")).max())
+        # and no further off than the CUDA-core GEMM it stands in for
+        simt = ajf.ajf_selftest_digit_gemm(0, precision, A, B, digits=False)
+        es = np.maximum(abs(simt.real - R[0]), abs(simt.imag - R[1])).astype(float)
+        assert np.linalg.norm(err) <= np.linalg.norm(es) or dist == "equal"
+
+
+@pytest.mark.gpu
+def test_fixed_arena_takes_plans_that_only_digits_outgrow():
+    """A plan over the 64 MiB of the no-allocation call because of its digit operands runs there with
+    CUDA-core GEMMs, and the context's own program is unchanged."""
+    inst = W.mid(0)
+    with ajf.Context(0) as c:
+        ajf.load_instance(c.handle, inst)
+        info = ajf.ajf_plan(c.handle, 1, trials=8)
+        assert info["n_tc_gemms"] > 0 and info["arena_bytes"] > 64 << 20
+        r = ajf.ajf_fidelity_alg1(c.handle)
+        n = ajf.ajf_fidelity_noalloc(c.handle, 1)
+        again = ajf.ajf_fidelity_alg1(c.handle)
+    assert abs(n["F"] - r["F"]) <= 1e-12 and again == r
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_budget_between_the_two_gemms_keeps_the_plan(precision):
+    """A memory budget that the CUDA-core GEMMs' plan meets is met, whatever the digit operands need."""
+    inst = W.mid(0)
+    with ajf.Context(-1) as c:
+        ajf.load_instance(c.handle, inst)
+        roomy = ajf.ajf_plan(c.handle, 2, precision=precision, trials=8)
+        assert roomy["n_tc_gemms"] > 0
+        ajf.ajf_check_plan(c.handle)
+        tight = ajf.ajf_plan(c.handle, 2, precision=precision, trials=8, mem_budget_bytes=0.96 * roomy["arena_bytes"])
+        ajf.ajf_check_plan(c.handle)
+        assert tight["n_tc_gemms"] == 0 and tight["arena_bytes"] <= 0.96 * roomy["arena_bytes"]
+        again = ajf.ajf_plan(c.handle, 2, precision=precision, trials=8)
+        assert again["n_tc_gemms"] > 0 and again["arena_bytes"] == roomy["arena_bytes"]
