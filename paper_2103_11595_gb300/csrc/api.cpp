@@ -1306,7 +1306,7 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
   pi.n_leaves = static_cast<int32_t>(c->net.leaf_labels.size());
   pi.n_open_bits = static_cast<int32_t>(c->net.open_labels.size());
   pi.planner_used = c->path.planner;
-  pi.n_launches = 3;  // leaves + final pass + final sum
+  pi.n_launches = P.final_blocks > 1 ? 3 : 2;  // leaves, final pass, and its sum over several blocks
   for (auto& ln : P.launches)
     pi.n_launches += (ln.kind == LK_SPLITK || ln.kind == LK_DOT || ln.row_exp > 0 ||
                       ((ln.kind == LK_GEMM_TC || ln.kind == LK_GEMM_DG) && ln.ksplit > 1)) ? 2 : 1;
@@ -2140,7 +2140,7 @@ ajf_status ajf_plan_launches(const ajf_ctx* c, ajf_launch_info* out, int cap, in
     if (ln.kind == LK_SPLITK || ln.kind == LK_DOT) add(2, 0, 0, 0, 0, 0, 0);  // the deterministic final-sum launch
   }
   add(6, 0, 0, 0, 0, 0, 0);
-  add(6, 0, 0, 0, 0, 0, 0);
+  if (c->prog.final_blocks > 1) add(6, 0, 0, 0, 0, 0, 0);
   *n = static_cast<int>(v.size());
   for (int i = 0; i < cap && i < static_cast<int>(v.size()); ++i) out[i] = v[i];
   return AJF_OK;

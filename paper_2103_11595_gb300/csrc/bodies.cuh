@@ -47,17 +47,49 @@ struct SyncBody {  // threads 0..kBodyThreads-1 of a larger block: named barrier
 
 __device__ __forceinline__ int nchunks(int nbits) { return (nbits + 7) >> 3; }
 
-// Fill `tab` (nchunks * 256 entries) for map `m`; all threads of the block participate.
+// Offsets that the 8 bits of chunk c of map `m` stand for (0: the bit addresses nothing).
+__device__ __forceinline__ void chunk_weights(const BitMap& m, int c, int64_t (&w)[8]) {
+  const uint32_t* words = reinterpret_cast<const uint32_t*>(m.pos);
+  const uint32_t p[2] = {words[2 * c], words[2 * c + 1]};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int pos = static_cast<int8_t>(p[i >> 2] >> (8 * (i & 3)));
+    w[i] = pos >= 0 ? int64_t(1) << (pos & 63) : 0;
+  }
+}
+__device__ __forceinline__ int64_t chunk_offset(const int64_t (&w)[8], int v) {
+  int64_t off = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) off += (v >> i) & 1 ? w[i] : 0;
+  return off;
+}
+
+// Fill `tab` (256 entries per chunk of 8 bits) for map `m`; the block's first kThreads threads
+// participate. A chunk's positions come in two words, and only the entries that its bits can index are
+// written (a step has often 2 to 6 bits).
+template <int kThreads = kBodyThreads>
 __device__ __forceinline__ void build_table(const BitMap& m, int64_t* tab) {
-  const int nc = nchunks(m.nbits);
-  for (int e = threadIdx.x; e < nc * 256; e += kBodyThreads) {
-    const int c = e >> 8, v = e & 255;
-    int64_t off = 0;
-    for (int i = 0; i < 8; ++i) {
-      const int bit = c * 8 + i;
-      if (bit < m.nbits && ((v >> i) & 1) && m.pos[bit] >= 0) off += int64_t(1) << m.pos[bit];
+  const int nbits = m.nbits, nc = nchunks(nbits);
+  for (int c = 0; c < nc; ++c) {
+    int64_t w[8];
+    chunk_weights(m, c, w);
+    const int bits = nbits - 8 * c < 8 ? nbits - 8 * c : 8;
+    for (int v = threadIdx.x; v < (1 << bits); v += kThreads) tab[(c << 8) | v] = chunk_offset(w, v);
+  }
+}
+// The tables of two maps over the same index (their instructions overlap).
+template <int kThreads = kBodyThreads>
+__device__ __forceinline__ void build_tables(const BitMap& m1, const BitMap& m2, int64_t* t1, int64_t* t2) {
+  const int nbits = m1.nbits, nc = nchunks(nbits);
+  for (int c = 0; c < nc; ++c) {
+    int64_t w1[8], w2[8];
+    chunk_weights(m1, c, w1);
+    chunk_weights(m2, c, w2);
+    const int bits = nbits - 8 * c < 8 ? nbits - 8 * c : 8;
+    for (int v = threadIdx.x; v < (1 << bits); v += kThreads) {
+      t1[(c << 8) | v] = chunk_offset(w1, v);
+      t2[(c << 8) | v] = chunk_offset(w2, v);
     }
-    tab[e] = off;
   }
 }
 
@@ -162,21 +194,57 @@ __device__ __forceinline__ void leaf_body(const LeafDev* leaves, const double* _
 
 // ------------------------------------------------------------------ small contractions
 
+// The step that owns block `block` of a launch (the last one with block0 <= block): 32 probes at a
+// time, so that a launch of up to 32 steps costs one load latency and one of up to 1024 two (a
+// binary search: up to ten, in series, at the head of every block). Whole warps.
 __device__ __forceinline__ int find_step(const StepDev* steps, int nsteps, int block) {
-  int lo = 0, hi = nsteps - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (steps[mid].block0 <= block) lo = mid; else hi = mid - 1;
+  const int lane = threadIdx.x & 31;
+  int lo = 0, n = nsteps;
+  while (n > 1) {
+    const int stride = (n + 31) >> 5, i = lane * stride;
+    const bool le = i < n && steps[lo + i].block0 <= block;
+    const int k = __popc(__ballot_sync(0xffffffffu, le)) - 1;
+    lo += k * stride;
+    n = n - k * stride < stride ? n - k * stride : stride;
   }
   return lo;
 }
 
-template <typename T, typename Acc, typename Sync>
+// Whether a factor vanishes, on the integer pipe.
+__device__ __forceinline__ bool is_zero(double x) {
+  return ((__double2hiint(x) << 1) | __double2loint(x)) == 0;
+}
+__device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
+// FP32 to FP64, exact, on the integer pipe (the conversion instruction takes the FP64 pipe as long as a
+// multiply-add does); subnormal and non-finite values through the instruction.
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x);
+  const bool zero = (b << 1) == 0;
+  if (((b >> 23) & 0xFFu) - 1u >= 254u && !zero) return static_cast<double>(x);
+  const uint32_t hi = (b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u);
+  return __hiloint2double(static_cast<int>(zero ? b : hi), static_cast<int>(b << 29));
+}
+
+// One thread per output. The FP64 pipe (2 multiply-adds per clock and SM) bounds large steps, latency
+// the many small ones (a warp's multiply-add takes 64 clocks, whatever its active lanes): the step's
+// descriptor is copied to shared memory in one go, the next four contracted indices are loaded while
+// four are multiplied, sums are fused multiply-adds (4 per complex product; a separate product and
+// sum takes 6), and entries of B that are
+// zero -- most of a CX or of a Kraus channel, and the same for whole warps, since B's bits are the
+// output's highest -- cost no FP64 instruction, real ones half. Measured per contracted index of a
+// warp: 920 -> 500 clocks (256 of them FP64); a launch of 16,384 outputs x 4 indices: 10.9 -> 6.3 thousand
+// clocks.
+template <typename T, typename Acc, typename Sync, int kThreads = kBodyThreads>
 __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, int nsteps, int total_blocks,
-                                           T* __restrict__ arena, int vb, int64_t* tab) {
+                                           T* __restrict__ arena, int vb, int64_t* tab, StepDev& st) {
   const int s = find_step(steps, nsteps, vb);
-  const StepDev& st = steps[s];
   const int end = (s + 1 < nsteps) ? steps[s + 1].block0 : total_blocks;
+  static_assert(sizeof(StepDev) % 4 == 0, "descriptor copy");
+  for (int i = threadIdx.x; i < static_cast<int>(sizeof(StepDev) / 4); i += kThreads)
+    reinterpret_cast<int32_t*>(&st)[i] = reinterpret_cast<const int32_t*>(&steps[s])[i];
+  Sync::sync();
+  if (int64_t(vb - st.block0) * kThreads >= int64_t(1) << st.rc) return;  // more blocks than outputs: all threads
   const int nb = end - st.block0;
   const int c_oa = nchunks(st.oa.nbits), c_ob = nchunks(st.ob.nbits);
   const int c_ka = nchunks(st.ka.nbits), c_kb = nchunks(st.kb.nbits);
@@ -184,23 +252,60 @@ __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, in
   int64_t* t_ob = t_oa + c_oa * 256;
   int64_t* t_ka = t_ob + c_ob * 256;
   int64_t* t_kb = t_ka + c_ka * 256;
-  build_table(st.oa, t_oa);
-  build_table(st.ob, t_ob);
-  build_table(st.ka, t_ka);
-  build_table(st.kb, t_kb);
+  build_tables<kThreads>(st.oa, st.ob, t_oa, t_ob);
+  build_tables<kThreads>(st.ka, st.kb, t_ka, t_kb);
   Sync::sync();
   const int64_t nout = int64_t(1) << st.rc, nk = int64_t(1) << st.rk;
+  const bool one_chunk = c_ka == 1;  // (no chunk, rk = 0: lookup gives 0)
   T* C = arena + st.c;
   with_operands(arena, st.a, st.fa, st.b, st.fb, [&](const auto* A, const auto* B) {
-    for (int64_t o = int64_t(vb - st.block0) * kBodyThreads + threadIdx.x; o < nout;
-         o += int64_t(nb) * kBodyThreads) {
-      const int64_t oa = lookup(t_oa, c_oa, o), ob = lookup(t_ob, c_ob, o);
+    using TA = typename std::remove_cv<typename std::remove_pointer<decltype(A)>::type>::type;
+    using TB = typename std::remove_cv<typename std::remove_pointer<decltype(B)>::type>::type;
+    for (int64_t o = int64_t(vb - st.block0) * kThreads + threadIdx.x; o < nout; o += int64_t(nb) * kThreads) {
+      const auto* Ao = A + lookup(t_oa, c_oa, o);
+      const auto* Bo = B + lookup(t_ob, c_ob, o);
       Acc re = 0, im = 0;
-      for (int64_t kk = 0; kk < nk; ++kk) {
-        const int64_t ia = oa + lookup(t_ka, c_ka, kk), ib = ob + lookup(t_kb, c_kb, kk);
-        const Acc ar = A[ia], ai = A[st.pa + ia], br = B[ib], bi = B[st.pb + ib];
-        re += ar * br - ai * bi;
-        im += ar * bi + ai * br;
+      TA ar[4], ai[4];
+      TB br[4], bi[4];
+      auto load = [&](int64_t kk) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (kk + j < nk) {
+            const int64_t ia = one_chunk ? t_ka[kk + j] : lookup(t_ka, c_ka, kk + j);
+            const int64_t ib = one_chunk ? t_kb[kk + j] : lookup(t_kb, c_kb, kk + j);
+            br[j] = Bo[ib];
+            bi[j] = Bo[st.pb + ib];
+            ar[j] = Ao[ia];
+            ai[j] = Ao[st.pa + ia];
+          }
+        }
+      };
+      load(0);
+      for (int64_t kk = 0; kk < nk; kk += 4) {
+        TA xr[4], xi[4];
+        TB yr[4], yi[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          xr[j] = ar[j];
+          xi[j] = ai[j];
+          yr[j] = br[j];
+          yi[j] = bi[j];
+        }
+        if (kk + 4 < nk) load(kk + 4);  // in flight while this group is multiplied
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (kk + j >= nk) break;
+          // (votes: a branch that the whole warp takes together needs no reconvergence)
+          const unsigned act = __activemask();
+          if (__any_sync(act, !is_zero(yr[j]))) {
+            re = fma(widen(xr[j]), widen(yr[j]), re);
+            im = fma(widen(xi[j]), widen(yr[j]), im);
+          }
+          if (__any_sync(act, !is_zero(yi[j]))) {
+            re = fma(-widen(xi[j]), widen(yi[j]), re);
+            im = fma(widen(xr[j]), widen(yi[j]), im);
+          }
+        }
       }
       C[o] = static_cast<T>(re);
       C[st.pc + o] = static_cast<T>(im);
@@ -238,9 +343,9 @@ __device__ __forceinline__ void splitk_body(const StepDev* __restrict__ steps, i
   with_operands(arena, st.a, st.fa, st.b, st.fb, [&](const auto* A, const auto* B) {
     for (int64_t kk = k0 + threadIdx.x; kk < k1; kk += kBodyThreads) {
       const int64_t ia = oa + lookup(t_ka, c_ka, kk), ib = ob + lookup(t_kb, c_kb, kk);
-      const double ar = A[ia], ai = A[st.pa + ia], br = B[ib], bi = B[st.pb + ib];
-      re += ar * br - ai * bi;
-      im += ar * bi + ai * br;
+      const double ar = widen(A[ia]), ai = widen(A[st.pa + ia]), br = widen(B[ib]), bi = widen(B[st.pb + ib]);
+      re = fma(-ai, bi, fma(ar, br, re));
+      im = fma(ai, br, fma(ar, bi, im));
     }
   });
   red_re[threadIdx.x] = re;
@@ -527,8 +632,8 @@ __device__ __forceinline__ void dot_body(const StepDev* __restrict__ steps, int 
             const int la = a_of_b[l];
             const int sl = la ^ ((la >> 5) & 31);
             const double ar = sre[sl], ai = sim[sl], br = cbr[q], bi = cbi[q];
-            re += ar * br - ai * bi;
-            im += ar * bi + ai * br;
+            re = fma(-ai, bi, fma(ar, br, re));
+            im = fma(ai, br, fma(ar, bi, im));
           }
         }
       }

@@ -16,6 +16,10 @@ namespace ajf {
 
 constexpr int kMaxBits = 48;
 
+// Threads of a small-step block (k_small). An SM adds FP64 products at 2 per clock, so a step of a few
+// hundred outputs is spread over as many SMs as its warps allow: 128 rather than 256 per block.
+constexpr int kSmallThreads = 128;
+
 // Map from the bits of an index to element offsets of one tensor: offset(idx) =
 // sum_i bit_i(idx) << pos[i] (pos < 0: the bit does not address this tensor). Evaluated on the
 // device through 8-bit lookup tables built in shared memory.

@@ -34,10 +34,11 @@ __global__ void __launch_bounds__(kBodyThreads) k_leaf(const LeafDev* leaves, co
 }
 
 template <typename T, typename Acc>
-__global__ void __launch_bounds__(kBodyThreads) k_small(const StepDev* __restrict__ steps, int nsteps,
-                                                        int total_blocks, T* __restrict__ arena) {
+__global__ void __launch_bounds__(kSmallThreads) k_small(const StepDev* __restrict__ steps, int nsteps,
+                                                         int total_blocks, T* __restrict__ arena) {
   extern __shared__ int64_t tab[];
-  small_body<T, Acc, SyncBlock>(steps, nsteps, total_blocks, arena, blockIdx.x, tab);
+  __shared__ StepDev st;
+  small_body<T, Acc, SyncBlock, kSmallThreads>(steps, nsteps, total_blocks, arena, blockIdx.x, tab, st);
 }
 
 template <typename T>
@@ -95,6 +96,19 @@ __global__ void __launch_bounds__(kBodyThreads) k_open(const FinalDev* __restric
 __global__ void k_final(const FinalDev* __restrict__ fd, const double2* __restrict__ scalars,
                         const double* __restrict__ partial, double* __restrict__ result) {
   if (threadIdx.x == 0) final_body(fd, scalars, partial, result);
+}
+
+// Both in one launch when one block covers the open tensor (always for Alg. II, whose result is the
+// product of scalars): one kernel less at the end of every evaluation's chain.
+template <typename T>
+__global__ void __launch_bounds__(kBodyThreads) k_open_final(const FinalDev* __restrict__ fd, const T* __restrict__ arena,
+                                                             const double2* __restrict__ scalars,
+                                                             double* __restrict__ traces, double* __restrict__ partial,
+                                                             double* __restrict__ result) {
+  extern __shared__ int64_t tab[];
+  __shared__ double red[kBodyThreads];
+  open_body<T, SyncBlock>(fd, arena, scalars, traces, partial, 0, 1, tab, red);
+  if (threadIdx.x == 0) final_body(fd, scalars, partial, result);  // partial[0]: this thread's own write
 }
 
 // ------------------------------------------------------------------ CUDA-core GEMM
@@ -344,7 +358,7 @@ cudaError_t launch_leaves(const LeafDev* d_leaves, int n, const double* d_in, vo
 cudaError_t launch_small(const StepDev* d_steps, int nsteps, int total_blocks, size_t smem, void* arena,
                          cudaStream_t s) {
   if (nsteps == 0) return cudaSuccess;
-  k_small<double, double><<<total_blocks, 256, smem, s>>>(d_steps, nsteps, total_blocks, static_cast<double*>(arena));
+  k_small<double, double><<<total_blocks, kSmallThreads, smem, s>>>(d_steps, nsteps, total_blocks, static_cast<double*>(arena));
   return cudaGetLastError();
 }
 
@@ -408,6 +422,11 @@ cudaError_t launch_gemm_simt(const void* A, const void* B, void* C, int64_t M, i
 cudaError_t launch_final(const FinalDev* d_fd, int open_bits_nchunks, int nblocks, const void* arena,
                          const double2* scalars, double* traces, double* partial, double* result, cudaStream_t s) {
   const size_t smem = size_t(open_bits_nchunks) * 256 * sizeof(int64_t);
+  if (nblocks == 1) {
+    k_open_final<double><<<1, kBodyThreads, smem, s>>>(d_fd, static_cast<const double*>(arena), scalars, traces, partial,
+                                                       result);
+    return cudaGetLastError();
+  }
   k_open<double><<<nblocks, 256, smem, s>>>(d_fd, static_cast<const double*>(arena), scalars, traces, partial);
   k_final<<<1, 32, 0, s>>>(d_fd, scalars, partial, result);
   return cudaGetLastError();
@@ -432,6 +451,7 @@ cudaError_t set_kernel_smem_limits() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_perm<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_perm<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_open<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_open_final<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
   return e;
 }
 

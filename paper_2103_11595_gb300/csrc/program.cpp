@@ -217,8 +217,9 @@ Program lower(const Network& net, const Path& path, int precision, size_t inputs
     } else {
       const bool a_big = la.size() >= lb.size();
       I.cls = (rc <= 12 && rk >= 10) ? C_SPLITK : C_SMALL;
-      I.a = st.a;
-      I.b = st.b;
+      // the larger operand is A: its bits are the output's lowest, so that a warp shares its B entries
+      I.a = a_big ? st.a : st.b;
+      I.b = a_big ? st.b : st.a;
       I.shared = sh;
       const auto& big = a_big ? fa : fb;
       const auto& small = a_big ? fb : fa;
@@ -420,7 +421,7 @@ Program lower(const Network& net, const Path& path, int precision, size_t inputs
         d.scalar_slot = -1;
         if (cls == C_SMALL) {
           const int64_t nout = int64_t(1) << d.rc;
-          blocks += static_cast<int>(std::min<int64_t>((nout + 255) / 256, 8192));
+          blocks += static_cast<int>(std::min<int64_t>((nout + kSmallThreads - 1) / kSmallThreads, 8192));
         } else if (cls == C_DOT) {
           // tile bits: the contracted bits on A's five lowest positions, then those on B's five
           // lowest, topped up from A's order (kl follows A's bit order)

@@ -70,7 +70,8 @@ __device__ __noinline__ void q_leaves(const QPhase& ph, int v) {
 }
 __device__ __noinline__ void q_small(const QPhase& ph, int v, uint8_t* smem) {
   small_body<double, double, SyncBody>(static_cast<const StepDev*>(ph.desc), ph.count, ph.nblocks,
-                                       reinterpret_cast<double*>(ph.base), v, reinterpret_cast<int64_t*>(smem));
+                                       reinterpret_cast<double*>(ph.base), v, reinterpret_cast<int64_t*>(smem),
+                                       *reinterpret_cast<StepDev*>(smem + kQArrays));
 }
 __device__ __noinline__ void q_splitk(const QPhase& ph, int v, uint8_t* smem) {
   double* red = reinterpret_cast<double*>(smem + kQArrays);

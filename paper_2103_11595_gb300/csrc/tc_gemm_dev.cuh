@@ -76,13 +76,10 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait: false (and status set) if the phase did not complete within limit_ns. The clock is
-// read only once the wait has failed many times: a read of the global timer takes longer than most
-// of a pipeline's waits (each of them used to pay one).
+// Bounded wait: false (and status set) if the phase did not complete within limit_ns.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long limit_ns, int* status,
                                           int code) {
-  for (int n = 0; n < 64; ++n)
-    if (mbar_try_wait(bar, parity)) return true;
+  if (mbar_try_wait(bar, parity)) return true;
   const unsigned long long t0 = globaltimer();
   for (uint32_t n = 1;; ++n) {
     if (mbar_try_wait(bar, parity)) return true;
