@@ -403,6 +403,15 @@ ajf_status prepare_tc_set(ajf_ctx* c, ajf_ctx::TcPrepSet* tc) {
   return AJF_OK;
 }
 
+// Whether a launch is so short (about 12 us by its algorithmic work) that its successor may start, and
+// wait, beside it (launch_chained).
+bool chain_early(const Launch& ln) {
+  const double us = ln.kind == LK_SMALL ? ln.flops / 0.8e6 + ln.bytes / 3e6  // FP64 pipe, HBM
+                                        : (ln.kind == LK_PERM || ln.kind == LK_DIGITS ? ln.bytes / 2e6
+                                                                                     : ln.flops / 20e6 + ln.bytes / 2e6);
+  return us < 12.0;
+}
+
 ajf_status enqueue_program(ajf_ctx* c, cudaStream_t s, ajf_ctx::TcPrepSet* tc = nullptr) {
   const Program& P = c->prog;
   char* base = c->arena;
@@ -434,25 +443,26 @@ ajf_status enqueue_program(ajf_ctx* c, cudaStream_t s, ajf_ctx::TcPrepSet* tc = 
         e = launch_dot(steps + ln.first, ln.count, ln.blocks, ln.smem, arena, partial, scalars, ln.op_f64 == 0, s);
         break;
       case LK_SMALL:
-        e = launch_small(steps + ln.first, ln.count, ln.blocks, ln.smem, arena, s);
+        e = launch_small(steps + ln.first, ln.count, ln.blocks, ln.smem, arena, s, chain_early(ln));
         break;
       case LK_SPLITK:
         e = launch_splitk(steps + ln.first, ln.count, ln.blocks, ln.smem, arena, partial, scalars, s);
         break;
       case LK_PERM:
-        e = launch_perm(perms + ln.first, ln.count, ln.blocks, ln.smem, arena, base, ln.op_f64 != 0, s);
+        e = launch_perm(perms + ln.first, ln.count, ln.blocks, ln.smem, arena, base, ln.op_f64 != 0, s, chain_early(ln));
         break;
       case LK_GEMM_SIMT:
         e = launch_gemm_simt(base + ln.a_off[0], base + ln.b_off[0], base + ln.c_off, ln.M, ln.N, ln.K, ln.op_f64 != 0,
                              s);
         break;
       case LK_GEMM_TC:
-        e = tc_gemm_run(tc->prep[li], s);
+        e = tc_gemm_run(tc->prep[li], s, chain_early(ln));
         break;
       case LK_DIGITS:
         e = cudaSuccess;
         if (ln.row_exp) e = launch_row_exp(perms + ln.first, ln.count, ln.row_exp, ln.smem, arena, base, s);
-        if (e == cudaSuccess) e = launch_digits(perms + ln.first, ln.count, ln.blocks, ln.smem, arena, base, ln.mode, s);
+        if (e == cudaSuccess) e = launch_digits(perms + ln.first, ln.count, ln.blocks, ln.smem, arena, base, ln.mode, s,
+                                                  chain_early(ln));
         break;
       case LK_GEMM_DG: {
         DgGemm g;
@@ -469,6 +479,7 @@ ajf_status enqueue_program(ajf_ctx* c, cudaStream_t s, ajf_ctx::TcPrepSet* tc = 
         g.ksplit = ln.ksplit;
         g.mode = ln.mode;
         g.wait_ns = kTcWaitNs;
+        g.early = chain_early(ln);
         e = launch_dg_gemm(g, s);
         break;
       }

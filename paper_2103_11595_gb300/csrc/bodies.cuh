@@ -43,6 +43,12 @@ struct SyncBody {  // threads 0..kBodyThreads-1 of a larger block: named barrier
   __device__ __forceinline__ static void sync() { asm volatile("bar.sync 1, %0;" ::"n"(kBodyThreads) : "memory"); }
 };
 
+// Chained launches (kernels.h, launch_chained): the successor may start / everything before is complete.
+__device__ __forceinline__ void chain_trigger(bool early) {
+  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------ offset tables
 
 __device__ __forceinline__ int nchunks(int nbits) { return (nbits + 7) >> 3; }
@@ -254,6 +260,7 @@ __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, in
   int64_t* t_kb = t_ka + c_ka * 256;
   build_tables<kThreads>(st.oa, st.ob, t_oa, t_ob);
   build_tables<kThreads>(st.ka, st.kb, t_ka, t_kb);
+  chain_wait();
   Sync::sync();
   const int64_t nout = int64_t(1) << st.rc, nk = int64_t(1) << st.rk;
   const bool one_chunk = c_ka == 1;  // (no chunk, rk = 0: lookup gives 0)
@@ -329,10 +336,9 @@ __device__ __forceinline__ void splitk_body(const StepDev* __restrict__ steps, i
   int64_t* t_ob = t_oa + c_oa * 256;
   int64_t* t_ka = t_ob + c_ob * 256;
   int64_t* t_kb = t_ka + c_ka * 256;
-  build_table(st.oa, t_oa);
-  build_table(st.ob, t_ob);
-  build_table(st.ka, t_ka);
-  build_table(st.kb, t_kb);
+  build_tables(st.oa, st.ob, t_oa, t_ob);
+  build_tables(st.ka, st.kb, t_ka, t_kb);
+  chain_wait();
   Sync::sync();
   const int64_t nk = int64_t(1) << st.rk;
   const int64_t chunk = (nk + st.nsplit - 1) / st.nsplit;
@@ -440,6 +446,7 @@ __device__ __forceinline__ void dot_body(const StepDev* __restrict__ steps, int 
       if ((kk >> st.tl[i]) & 1) la |= 1 << i;
     a_of_b[l] = static_cast<uint16_t>(la);
   }
+  chain_wait();
   Sync::sync();
   const int64_t ntiles = int64_t(1) << (st.rk - ntl);
   // vector form: both operands FP32 with their two lowest positions the tile's two lowest bits in
@@ -1006,6 +1013,7 @@ __device__ __forceinline__ void perm_body(const PermDev* __restrict__ perms, con
   int64_t* t_k = tab + c_r * 256;
   build_table(p.rows, t_r);
   build_table(p.cols, t_k);
+  chain_wait();
   Sync::sync();
   if constexpr (sizeof(S) == 4) {
     if (p.mode == OPM_BF16X3 && p.rbits >= 5 && p.kbits >= 6) {

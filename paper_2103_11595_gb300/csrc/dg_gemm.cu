@@ -124,6 +124,7 @@ __device__ __forceinline__ void row_exp_body(const PermDev& p, const S* __restri
   int64_t* t_k = tab + c_r * 256;
   build_table(p.rows, t_r);
   build_table(p.cols, t_k);
+  chain_wait();
   __syncthreads();
   const int64_t R = int64_t(1) << p.rbits;
   const int TR = 1 << p.tr;
@@ -211,6 +212,7 @@ __device__ __forceinline__ void digits_body(const PermDev& p, const S* __restric
   int64_t* t_k = tab + c_r * 256;
   build_table(p.rows, t_r);
   build_table(p.cols, t_k);
+  chain_wait();
   __syncthreads();
   const int64_t R = int64_t(1) << p.rbits, K = int64_t(1) << p.kbits;
   const int kt_bits = p.kbits - p.tk;              // log2 of the tiles along K
@@ -317,7 +319,9 @@ __device__ __forceinline__ void digits_body(const PermDev& p, const S* __restric
 
 template <int T>
 __global__ void __launch_bounds__(kBodyThreads, 3) k_digits(const PermDev* __restrict__ perms,
-                                                            const double* __restrict__ arena, char* __restrict__ base) {
+                                                            const double* __restrict__ arena, char* __restrict__ base,
+                                                            bool early) {
+  chain_trigger(early);
   extern __shared__ int64_t tab[];
   __shared__ __align__(16) double tile[2 * kTileElems];
   const PermDev& p = perms[blockIdx.y];
@@ -354,6 +358,7 @@ struct DgParams {
   int32_t nty, ntx, group;           // tiles along Y and X, raster group
   int32_t yrows;                     // rows of a Y row block
   uint32_t idesc;
+  int32_t early;
   unsigned long long wait_ns;
 };
 
@@ -446,6 +451,7 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem, uint32_t alo, uint32_t bl
 
 template <int BC, int T, int PACK, typename Out>
 __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__ DgParams p) {
+  chain_trigger(p.early != 0);
   constexpr int kLevels = T == 6 ? 7 : 4;
   constexpr int COLS = BC / 4;                 // columns per epilogue thread
   constexpr int CH = COLS < 16 ? COLS : 16;    // columns per TMEM load
@@ -482,6 +488,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = __shfl_sync(0xffffffffu, *sh.tmem_slot, 0);
+  chain_wait();
 
   // work item wi: tile wi % tiles of K split wi / tiles; `group` Y blocks sweep the X blocks together
   const uint32_t tiles = static_cast<uint32_t>(p.nty) * static_cast<uint32_t>(p.ntx);
@@ -767,6 +774,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
 template <typename Out>
 __global__ void __launch_bounds__(kBodyThreads) k_dg_split_sum(const double* __restrict__ W, int ksplit, int64_t n,
                                                                Out* __restrict__ C) {
+  chain_wait();
   for (int64_t i = int64_t(blockIdx.x) * kBodyThreads + threadIdx.x; i < n; i += int64_t(gridDim.x) * kBodyThreads) {
     double s = W[i];
     for (int k = 1; k < ksplit; ++k) s += W[k * n + i];
@@ -815,8 +823,8 @@ cudaError_t run_dg(DgParams& p, cudaStream_t s) {
   // as few CTAs as keep the number of rounds at its minimum (the SMs left over run other streams)
   const int64_t work = int64_t(p.nty) * p.ntx * p.ksplit;
   const int64_t rounds = (work + sms - 1) / sms;
-  k_dg_gemm<BC, T, PACK, Out><<<static_cast<unsigned>((work + rounds - 1) / rounds), kThreads, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_chained(k_dg_gemm<BC, T, PACK, Out>, dim3(static_cast<unsigned>((work + rounds - 1) / rounds)), kThreads, smem,
+                        s, p);
 }
 
 template <int BC, int T, typename Out>
@@ -861,19 +869,14 @@ int dg_gemm_splits(int64_t M, int64_t N, int64_t K) {
 
 cudaError_t launch_row_exp(const PermDev* d_perms, int nperm, int grid_x, size_t smem, const void* arena, void* base,
                            cudaStream_t s) {
-  k_row_exp<<<dim3(grid_x, nperm), kBodyThreads, smem, s>>>(d_perms, static_cast<const double*>(arena),
-                                                            static_cast<char*>(base));
-  return cudaGetLastError();
+  return launch_chained(k_row_exp, dim3(grid_x, nperm), kBodyThreads, smem, s, d_perms, static_cast<const double*>(arena),
+                        static_cast<char*>(base));
 }
 
 cudaError_t launch_digits(const PermDev* d_perms, int nperm, int grid_x, size_t smem, const void* arena, void* base,
-                          int mode, cudaStream_t s) {
-  const dim3 grid(grid_x, nperm);
-  if (mode == OPM_DIG6)
-    k_digits<6><<<grid, kBodyThreads, smem, s>>>(d_perms, static_cast<const double*>(arena), static_cast<char*>(base));
-  else
-    k_digits<4><<<grid, kBodyThreads, smem, s>>>(d_perms, static_cast<const double*>(arena), static_cast<char*>(base));
-  return cudaGetLastError();
+                          int mode, cudaStream_t s, bool early) {
+  return launch_chained(mode == OPM_DIG6 ? k_digits<6> : k_digits<4>, dim3(grid_x, nperm), kBodyThreads, smem, s, d_perms,
+                        static_cast<const double*>(arena), static_cast<char*>(base), early);
 }
 
 cudaError_t launch_dg_gemm(const DgGemm& g, cudaStream_t s) {
@@ -900,6 +903,7 @@ cudaError_t launch_dg_gemm(const DgGemm& g, cudaStream_t s) {
   if (p.pack == 0) p.sh0 = std::min(p.sh0, 39);
   p.yrows = static_cast<int32_t>(block_rows(g.N));
   p.wait_ns = g.wait_ns;
+  p.early = g.early ? 1 : 0;
   cudaError_t e;
   if (g.mode == OPM_DIG6) e = run_dg_t<6, double>(p, s);
   else e = run_dg_t<4, float>(p, s);
@@ -907,10 +911,10 @@ cudaError_t launch_dg_gemm(const DgGemm& g, cudaStream_t s) {
   const int64_t n = g.M * g.N;
   const unsigned blocks = static_cast<unsigned>(std::min<int64_t>((n + 255) / 256, 4096));
   if (g.mode == OPM_DIG6)
-    k_dg_split_sum<double><<<blocks, kBodyThreads, 0, s>>>(g.ws, g.ksplit, n, static_cast<double*>(g.C));
-  else
-    k_dg_split_sum<float><<<blocks, kBodyThreads, 0, s>>>(g.ws, g.ksplit, n, static_cast<float*>(g.C));
-  return cudaGetLastError();
+    return launch_chained(k_dg_split_sum<double>, dim3(blocks), kBodyThreads, size_t(0), s, g.ws, g.ksplit, n,
+                          static_cast<double*>(g.C));
+  return launch_chained(k_dg_split_sum<float>, dim3(blocks), kBodyThreads, size_t(0), s, g.ws, g.ksplit, n,
+                        static_cast<float*>(g.C));
 }
 
 cudaError_t set_dg_smem_limits() {

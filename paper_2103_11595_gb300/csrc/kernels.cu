@@ -35,9 +35,10 @@ __global__ void __launch_bounds__(kBodyThreads) k_leaf(const LeafDev* leaves, co
 
 template <typename T, typename Acc>
 __global__ void __launch_bounds__(kSmallThreads) k_small(const StepDev* __restrict__ steps, int nsteps,
-                                                         int total_blocks, T* __restrict__ arena) {
+                                                         int total_blocks, T* __restrict__ arena, bool early) {
   extern __shared__ int64_t tab[];
   __shared__ StepDev st;
+  chain_trigger(early);
   small_body<T, Acc, SyncBlock, kSmallThreads>(steps, nsteps, total_blocks, arena, blockIdx.x, tab, st);
 }
 
@@ -64,6 +65,7 @@ __global__ void __launch_bounds__(kBodyThreads) k_splitk_done(const StepDev* __r
                                                               const double2* __restrict__ partial,
                                                               T* __restrict__ arena, double2* __restrict__ scalars) {
   (void)nsteps;
+  chain_wait();
   __shared__ double red_re[kBodyThreads], red_im[kBodyThreads];
   splitk_done_body<T, SyncBlock>(steps, partial, arena, scalars, blockIdx.x, red_re, red_im);
 }
@@ -73,9 +75,11 @@ __global__ void __launch_bounds__(kBodyThreads) k_splitk_done(const StepDev* __r
 // the FP64 operand mode, FP32 otherwise).
 template <typename S>
 __global__ void __launch_bounds__(kBodyThreads, 4) k_perm(const PermDev* __restrict__ perms,
-                                                       const double* __restrict__ arena, char* __restrict__ base) {
+                                                       const double* __restrict__ arena, char* __restrict__ base,
+                                                       bool early) {
   extern __shared__ int64_t tab[];
   __shared__ PermSmem<S> sm;
+  chain_trigger(early);
   if constexpr (sizeof(S) == 4) {
     __shared__ PermSmem<float> sm2;  // second tile buffer of the six-product split's copy pipeline
     perm_body<S, SyncBlock>(perms, arena, base, blockIdx.x, gridDim.x, blockIdx.y, tab, sm, &sm2);
@@ -90,11 +94,13 @@ __global__ void __launch_bounds__(kBodyThreads) k_open(const FinalDev* __restric
                                                        double* __restrict__ traces, double* __restrict__ partial) {
   extern __shared__ int64_t tab[];
   __shared__ double red[kBodyThreads];
+  chain_wait();
   open_body<T, SyncBlock>(fd, arena, scalars, traces, partial, blockIdx.x, gridDim.x, tab, red);
 }
 
 __global__ void k_final(const FinalDev* __restrict__ fd, const double2* __restrict__ scalars,
                         const double* __restrict__ partial, double* __restrict__ result) {
+  chain_wait();
   if (threadIdx.x == 0) final_body(fd, scalars, partial, result);
 }
 
@@ -107,6 +113,7 @@ __global__ void __launch_bounds__(kBodyThreads) k_open_final(const FinalDev* __r
                                                              double* __restrict__ result) {
   extern __shared__ int64_t tab[];
   __shared__ double red[kBodyThreads];
+  chain_wait();
   open_body<T, SyncBlock>(fd, arena, scalars, traces, partial, 0, 1, tab, red);
   if (threadIdx.x == 0) final_body(fd, scalars, partial, result);  // partial[0]: this thread's own write
 }
@@ -356,18 +363,20 @@ cudaError_t launch_leaves(const LeafDev* d_leaves, int n, const double* d_in, vo
 }
 
 cudaError_t launch_small(const StepDev* d_steps, int nsteps, int total_blocks, size_t smem, void* arena,
-                         cudaStream_t s) {
+                         cudaStream_t s, bool early) {
   if (nsteps == 0) return cudaSuccess;
-  k_small<double, double><<<total_blocks, kSmallThreads, smem, s>>>(d_steps, nsteps, total_blocks, static_cast<double*>(arena));
-  return cudaGetLastError();
+  return launch_chained(k_small<double, double>, dim3(total_blocks), kSmallThreads, smem, s, d_steps, nsteps, total_blocks,
+                        static_cast<double*>(arena), early);
 }
 
 cudaError_t launch_splitk(const StepDev* d_steps, int nsteps, int total_blocks, size_t smem, void* arena,
                           double2* partial, double2* scalars, cudaStream_t s) {
   if (nsteps == 0) return cudaSuccess;
-  k_splitk<double><<<total_blocks, 256, smem, s>>>(d_steps, nsteps, static_cast<const double*>(arena), partial);
-  k_splitk_done<double><<<nsteps, 256, 0, s>>>(d_steps, nsteps, partial, static_cast<double*>(arena), scalars);
-  return cudaGetLastError();
+  const cudaError_t e = launch_chained(k_splitk<double>, dim3(total_blocks), 256u, smem, s, d_steps, nsteps,
+                                       static_cast<const double*>(arena), partial);
+  if (e != cudaSuccess) return e;
+  return launch_chained(k_splitk_done<double>, dim3(nsteps), 256u, size_t(0), s, d_steps, nsteps, partial,
+                        static_cast<double*>(arena), scalars);
 }
 
 bool dot_staged(const StepDev& st, bool f32_products) { return f32_products && st.fa && st.fb && st.ntl == 10; }
@@ -383,26 +392,21 @@ size_t dot_smem_bytes(const StepDev& st, bool f32_products) {
 cudaError_t launch_dot(const StepDev* d_steps, int nsteps, int total_blocks, size_t smem, const void* arena,
                        double2* partial, double2* scalars, bool f32_products, cudaStream_t s) {
   if (nsteps == 0) return cudaSuccess;
-  if (f32_products)
-    k_dot<double, true><<<total_blocks, 256, smem, s>>>(d_steps, nsteps, static_cast<const double*>(arena), partial);
-  else
-    k_dot<double, false><<<total_blocks, 256, smem, s>>>(d_steps, nsteps, static_cast<const double*>(arena), partial);
-  k_splitk_done<double><<<nsteps, 256, 0, s>>>(d_steps, nsteps, partial, static_cast<double*>(const_cast<void*>(arena)),
-                                               scalars);
-  return cudaGetLastError();
+  const cudaError_t e = launch_chained(f32_products ? k_dot<double, true> : k_dot<double, false>, dim3(total_blocks), 256u,
+                                       smem, s, d_steps, nsteps, static_cast<const double*>(arena), partial);
+  if (e != cudaSuccess) return e;
+  return launch_chained(k_splitk_done<double>, dim3(nsteps), 256u, size_t(0), s, d_steps, nsteps, partial,
+                        static_cast<double*>(const_cast<void*>(arena)), scalars);
 }
 
 cudaError_t launch_perm(const PermDev* d_perms, int nperm, int grid_x, size_t smem, const void* arena, void* base,
-                        bool op_f64, cudaStream_t s) {
+                        bool op_f64, cudaStream_t s, bool early) {
   if (nperm == 0) return cudaSuccess;
   dim3 grid(grid_x, nperm);
   // the operand format (FP64 or a reduced one) is in each PermDev, and every PermDev of one launch
   // has the same one; each source is complex128, or complex64 when a reduced-precision GEMM made it
-  if (op_f64)
-    k_perm<double><<<grid, 256, smem, s>>>(d_perms, static_cast<const double*>(arena), static_cast<char*>(base));
-  else
-    k_perm<float><<<grid, 256, smem, s>>>(d_perms, static_cast<const double*>(arena), static_cast<char*>(base));
-  return cudaGetLastError();
+  return launch_chained(op_f64 ? k_perm<double> : k_perm<float>, grid, 256u, smem, s, d_perms,
+                        static_cast<const double*>(arena), static_cast<char*>(base), early);
 }
 
 cudaError_t launch_gemm_simt(const void* A, const void* B, void* C, int64_t M, int64_t N, int64_t K, bool f64,
@@ -422,14 +426,12 @@ cudaError_t launch_gemm_simt(const void* A, const void* B, void* C, int64_t M, i
 cudaError_t launch_final(const FinalDev* d_fd, int open_bits_nchunks, int nblocks, const void* arena,
                          const double2* scalars, double* traces, double* partial, double* result, cudaStream_t s) {
   const size_t smem = size_t(open_bits_nchunks) * 256 * sizeof(int64_t);
-  if (nblocks == 1) {
-    k_open_final<double><<<1, kBodyThreads, smem, s>>>(d_fd, static_cast<const double*>(arena), scalars, traces, partial,
-                                                       result);
-    return cudaGetLastError();
-  }
-  k_open<double><<<nblocks, 256, smem, s>>>(d_fd, static_cast<const double*>(arena), scalars, traces, partial);
-  k_final<<<1, 32, 0, s>>>(d_fd, scalars, partial, result);
-  return cudaGetLastError();
+  const double* in = static_cast<const double*>(arena);
+  if (nblocks == 1)
+    return launch_chained(k_open_final<double>, dim3(1), kBodyThreads, smem, s, d_fd, in, scalars, traces, partial, result);
+  const cudaError_t e = launch_chained(k_open<double>, dim3(nblocks), kBodyThreads, smem, s, d_fd, in, scalars, traces, partial);
+  if (e != cudaSuccess) return e;
+  return launch_chained(k_final, dim3(1), 32u, size_t(0), s, d_fd, scalars, partial, result);
 }
 
 size_t step_table_bytes(const StepDev& st) {

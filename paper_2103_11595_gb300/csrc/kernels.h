@@ -8,6 +8,28 @@ namespace ajf {
 
 cudaError_t set_kernel_smem_limits();
 
+// Launches of a program's chain of dependent kernels. Every kernel of the chain is launched with
+// programmatic stream serialization and waits (griddepcontrol.wait) before its first access to what
+// other kernels read or write, so its launch latency, descriptor loads and offset tables overlap the
+// end of the kernel before it. `early`: the kernel lets its successor start at once; set for short
+// kernels only (chain_early), because a successor that waits for long holds shared memory and warps that
+// other streams could use.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                           Args... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // Fixed device arena (static_arena.cu) for evaluations that allocate nothing: its size, and its
 // device address on `device`, which must be the current device (cudaErrorInvalidDevice otherwise).
 constexpr size_t kStaticArenaBytes = size_t(64) << 20;
@@ -16,12 +38,13 @@ size_t step_table_bytes(const StepDev& st);
 size_t perm_table_bytes(const PermDev& p);
 
 cudaError_t launch_leaves(const LeafDev* d_leaves, int n, const double* d_in, void* arena, cudaStream_t s);
-cudaError_t launch_small(const StepDev* d_steps, int nsteps, int total_blocks, size_t smem, void* arena, cudaStream_t s);
+cudaError_t launch_small(const StepDev* d_steps, int nsteps, int total_blocks, size_t smem, void* arena, cudaStream_t s,
+                         bool early = false);
 cudaError_t launch_splitk(const StepDev* d_steps, int nsteps, int total_blocks, size_t smem, void* arena,
                           double2* partial, double2* scalars, cudaStream_t s);
 // op_f64: the operands are FP64 (staged in FP64); otherwise every format is staged in FP32.
 cudaError_t launch_perm(const PermDev* d_perms, int nperm, int grid_x, size_t smem, const void* arena, void* base,
-                        bool op_f64, cudaStream_t s);
+                        bool op_f64, cudaStream_t s, bool early = false);
 // Tiled FP64 full contraction (k_dot) of steps with a scalar result, then the partial-sum pass.
 // The tiled dot's staged form (FP32 operands, FP32 products): the step qualifies on the host side;
 // the kernel also checks the operands' bit positions and alignment and otherwise falls back.
@@ -51,7 +74,7 @@ int dg_gemm_splits(int64_t M, int64_t N, int64_t K);
 cudaError_t launch_row_exp(const PermDev* d_perms, int nperm, int grid_x, size_t smem, const void* arena, void* base,
                            cudaStream_t s);
 cudaError_t launch_digits(const PermDev* d_perms, int nperm, int grid_x, size_t smem, const void* arena, void* base,
-                          int mode, cudaStream_t s);
+                          int mode, cudaStream_t s, bool early = false);
 struct DgGemm {
   const void* x = nullptr;   // X digits (M rows: embedded complex rows), Y digits (N rows)
   const void* y = nullptr;
@@ -62,6 +85,7 @@ struct DgGemm {
   int* status = nullptr;
   int64_t M = 0, N = 0, K = 0;
   int ksplit = 1, mode = OPM_DIG6;
+  bool early = false;        // see launch_chained
   unsigned long long wait_ns = 0;  // bound of every device-side wait
 };
 cudaError_t launch_dg_gemm(const DgGemm& g, cudaStream_t s);
@@ -80,7 +104,7 @@ int tc_gemm_splits(int64_t M, int64_t N, int64_t K, int kind);
 // enqueueing it later costs one kernel launch (two with a K split) and no host set-up.
 struct TcPrepared {
   alignas(64) unsigned char params[1024];  // the kernel's parameter block
-  void (*run)(const void* params, unsigned grid, size_t smem, cudaStream_t s) = nullptr;
+  cudaError_t (*run)(const void* params, unsigned grid, size_t smem, cudaStream_t s, bool early) = nullptr;
   unsigned grid = 0;
   size_t smem = 0;
   int ksplit = 1;
@@ -92,7 +116,7 @@ struct TcPrepared {
 cudaError_t tc_gemm_prepare(TcPrepared* t, char* base, const int64_t* a_off, const int64_t* b_off, int terms,
                             float* C, int64_t M, int64_t N, int64_t K, int kind, float* ws, int ksplit,
                             int* d_status, unsigned long long wait_ns, int stall_loads);
-cudaError_t tc_gemm_run(const TcPrepared& t, cudaStream_t s);
+cudaError_t tc_gemm_run(const TcPrepared& t, cudaStream_t s, bool early = false);
 // Bound of every device-side wait in the GEMM and the step interpreter (nanoseconds).
 constexpr unsigned long long kTcWaitNs = 2000000000ull;
 // Persistent step interpreter (queue.cu): one launch of `blocks` blocks (at most one per SM) runs

@@ -68,7 +68,8 @@ namespace {
 using namespace tc;
 
 template <int BN, int kKind>
-__global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__ TcParams p) {
+__global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__ TcParams p, bool early) {
+  chain_trigger(early);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5;
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   sh.tmem = *tmem_slot;
+  chain_wait();
   TcRing ring;
   const uint32_t nwork = static_cast<uint32_t>(p.tiles) * static_cast<uint32_t>(p.ksplit);
   tc_gemm_items<BN, kKind>(p, blockIdx.x, nwork, gridDim.x, sh, ring);
@@ -146,8 +148,8 @@ int sm_count() {
 }
 
 template <int BN, int KIND>
-void run_tile(const void* params, unsigned grid, size_t smem, cudaStream_t s) {
-  k_gemm_tc<BN, KIND><<<grid, kThreads, smem, s>>>(*static_cast<const TcParams*>(params));
+cudaError_t run_tile(const void* params, unsigned grid, size_t smem, cudaStream_t s, bool early) {
+  return launch_chained(k_gemm_tc<BN, KIND>, dim3(grid), kThreads, smem, s, *static_cast<const TcParams*>(params), early);
 }
 
 // Fill the tile geometry of `p` and the launch shape of `t` (host only; nothing is enqueued).
@@ -234,6 +236,7 @@ namespace {
 // C[i] = sum over splits s (in order) of W[s][i] (compensated FP32 sum)
 __global__ void __launch_bounds__(kBodyThreads) k_split_sum(const float* __restrict__ W, int ksplit, int64_t n,
                                                             float* __restrict__ C) {
+  chain_wait();
   split_sum_body(W, ksplit, n, C, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x));
 }
 
@@ -296,14 +299,12 @@ cudaError_t tc_gemm_prepare(TcPrepared* t, char* base, const int64_t* a_off, con
   return cudaSuccess;
 }
 
-cudaError_t tc_gemm_run(const TcPrepared& t, cudaStream_t s) {
+cudaError_t tc_gemm_run(const TcPrepared& t, cudaStream_t s, bool early) {
   if (!t.ready) return cudaErrorInvalidValue;
-  t.run(t.params, t.grid, t.smem, s);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = t.run(t.params, t.grid, t.smem, s, early);
   if (e != cudaSuccess || t.ksplit == 1) return e;
   const int64_t blocks = (t.n + 255) / 256 < 4096 ? (t.n + 255) / 256 : 4096;
-  k_split_sum<<<static_cast<unsigned>(blocks), kBodyThreads, 0, s>>>(t.ws, t.ksplit, t.n, t.C);
-  return cudaGetLastError();
+  return launch_chained(k_split_sum, dim3(static_cast<unsigned>(blocks)), kBodyThreads, size_t(0), s, t.ws, t.ksplit, t.n, t.C);
 }
 
 cudaError_t launch_gemm_tc(char* base, const int64_t* a_off, const int64_t* b_off, int terms, float* C, int64_t M,
