@@ -200,6 +200,21 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_gemm_simt(const T* __
 
 // ------------------------------------------------------------------ persistent kernel
 
+// Offsets of one map for the indices of a small network's step: the first 8 bits from weights held in
+// registers (two loads), any beyond bit by bit.
+struct MapOffset {
+  int64_t w[8];
+  int nbits;
+  const BitMap* m;
+  __device__ __forceinline__ explicit MapOffset(const BitMap& map) : nbits(map.nbits), m(&map) { chunk_weights(map, 0, w); }
+  __device__ __forceinline__ int64_t operator()(int64_t idx) const {
+    if (nbits == 0) return 0;
+    int64_t off = chunk_offset(w, static_cast<int>(idx & 255));
+    for (int i = 8; i < nbits; ++i)
+      if (((idx >> i) & 1) && m->pos[i] >= 0) off += int64_t(1) << m->pos[i];
+    return off;
+  }
+};
 // offset(idx) = sum over the map's bits set in idx of 2^pos (bits with pos < 0 address nothing)
 __device__ __forceinline__ int64_t map_offset(const BitMap& m, int64_t idx) {
   int64_t off = 0;
@@ -208,19 +223,16 @@ __device__ __forceinline__ int64_t map_offset(const BitMap& m, int64_t idx) {
   return off;
 }
 
-// First local index handled by this thread when the flat index space continues from `base`
-// (thread t takes the flat indices congruent to t modulo the block size).
-__device__ __forceinline__ int64_t first_local(int64_t base, int unit, int nunits) {
-  return ((unit - base % nunits) % nunits + nunits) % nunits;
-}
-
 // One thread block per network runs the network's whole program: leaves, every step in level
 // order (one block barrier per level), the FP64 trace and F. The work region (all tensors) is
-// kept in shared memory when it fits (job.smem), otherwise it stays in the arena. Steps of one
-// level are independent; a level's outputs are spread over the threads (LK_SMALL: a thread per
-// output element; LK_SPLITK: a warp per output element, lanes along the contracted index,
-// summed in a fixed shuffle order).
-__global__ void __launch_bounds__(256) k_persistent(const InterpJob* __restrict__ jobs,
+// kept in shared memory when it fits (job.smem), otherwise it stays in the arena. Latency bound: a
+// few hundred multiply-adds per level. So the block's warps share out a level's leaves and steps
+// instead of walking all of them in step -- reading every descriptor of a level in every thread, one
+// load latency (700 clocks) after the other, was most of the kernel's time: a level's work is cut
+// into warp units (LK_SMALL: 32 outputs, one per lane; LK_SPLITK: one output, lanes along the
+// contracted index, summed in a fixed shuffle order), whose owners come from a scan over the steps'
+// sizes, 32 descriptors per load.
+__global__ void __launch_bounds__(256, 2) k_persistent(const InterpJob* __restrict__ jobs,
                                                     const InterpOp* __restrict__ ops) {
   extern __shared__ double swork[];
   __shared__ double red[256];
@@ -229,60 +241,78 @@ __global__ void __launch_bounds__(256) k_persistent(const InterpJob* __restrict_
   double* W = J.smem ? swork : arena;
   const int64_t w0 = J.smem ? J.work0 : 0;
   const int tid = threadIdx.x, nt = blockDim.x;
+  const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
 
   // leaves
   {
     const LeafDev* leaves = reinterpret_cast<const LeafDev*>(J.base + J.off_leaves);
     const double* in = reinterpret_cast<const double*>(J.base + J.off_inputs);
-    int64_t base = 0;
-    for (int l = 0; l < J.n_leaves; ++l) {
+    for (int l = warp; l < J.n_leaves; l += nw) {
       const LeafDev L = leaves[l];
       const int64_t n = int64_t(1) << L.bits;
-      for (int64_t e = first_local(base, tid, nt); e < n; e += nt) {
+      for (int64_t e = lane; e < n; e += 32) {
         double re, im;
         leaf_value(L, in, leaf_full_index(L, e), re, im);
         W[L.off - w0 + e] = re;
         W[L.off - w0 + L.plane + e] = im;
       }
-      base += n;
     }
   }
   __syncthreads();
 
   const StepDev* steps = reinterpret_cast<const StepDev*>(J.base + J.off_steps);
   double2* scalars = reinterpret_cast<double2*>(J.base + J.off_scalars);
-  const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
   for (int q = 0; q < J.n_ops; ++q) {
     const InterpOp op = ops[J.op0 + q];
-    int64_t base = 0;
-    for (int s = op.first; s < op.first + op.count; ++s) {
-      const StepDev& st = steps[s];
-      const int64_t nout = int64_t(1) << st.rc, nk = int64_t(1) << st.rk;
-      const double* A = W + (st.a - w0);
-      const double* B = W + (st.b - w0);
-      if (op.kind == 0) {
-        double* C = W + (st.c - w0);
-        for (int64_t o = first_local(base, tid, nt); o < nout; o += nt) {
-          const int64_t oa = map_offset(st.oa, o), ob = map_offset(st.ob, o);
-          double re = 0, im = 0;
-          for (int64_t kk = 0; kk < nk; ++kk) {
-            const int64_t ia = oa + map_offset(st.ka, kk), ib = ob + map_offset(st.kb, kk);
-            const double ar = A[ia], ai = A[st.pa + ia], br = B[ib], bi = B[st.pb + ib];
-            re += ar * br - ai * bi;
-            im += ar * bi + ai * br;
+    int64_t first = 0;  // units of the level so far, modulo the warps: the next step's units continue there
+    for (int s0 = 0; s0 < op.count; s0 += 32) {
+      // units of steps s0 .. s0 + 31 (one per lane) and their exclusive prefix
+      int64_t units = 0;
+      if (s0 + lane < op.count) {
+        const int rc = steps[op.first + s0 + lane].rc;
+        units = op.kind == 0 ? (rc > 5 ? int64_t(1) << (rc - 5) : 1) : int64_t(1) << rc;
+      }
+      int64_t incl = units;
+#pragma unroll
+      for (int w = 1; w < 32; w <<= 1) {
+        const int64_t v = __shfl_up_sync(0xffffffffu, incl, w);
+        if (lane >= w) incl += v;
+      }
+      const int64_t total = __shfl_sync(0xffffffffu, incl, 31), excl = incl - units;
+      for (int64_t u = (warp - first % nw + nw) % nw; u < total; u += nw) {
+        const int k = __popc(__ballot_sync(0xffffffffu, units > 0 && excl <= u)) - 1;
+        const int64_t local = u - __shfl_sync(0xffffffffu, excl, k);
+        const StepDev& st = steps[op.first + s0 + k];
+        const int64_t nout = int64_t(1) << st.rc, nk = int64_t(1) << st.rk;
+        const double* A = W + (st.a - w0);
+        const double* B = W + (st.b - w0);
+        const MapOffset ka(st.ka), kb(st.kb);
+        if (op.kind == 0) {
+          const int64_t o = local * 32 + lane;
+          if (o < nout) {
+            const double* Ao = A + MapOffset(st.oa)(o);
+            const double* Bo = B + MapOffset(st.ob)(o);
+            double re = 0, im = 0;
+            for (int64_t kk = 0; kk < nk; ++kk) {
+              const int64_t ia = ka(kk), ib = kb(kk);
+              const double ar = Ao[ia], ai = Ao[st.pa + ia], br = Bo[ib], bi = Bo[st.pb + ib];
+              re = fma(-ai, bi, fma(ar, br, re));
+              im = fma(ai, br, fma(ar, bi, im));
+            }
+            double* C = W + (st.c - w0);
+            C[o] = re;
+            C[st.pc + o] = im;
           }
-          C[o] = re;
-          C[st.pc + o] = im;
-        }
-      } else {
-        for (int64_t o = first_local(base, warp, nw); o < nout; o += nw) {
-          const int64_t oa = map_offset(st.oa, o), ob = map_offset(st.ob, o);
+        } else {
+          const int64_t o = local;
+          const double* Ao = A + MapOffset(st.oa)(o);
+          const double* Bo = B + MapOffset(st.ob)(o);
           double re = 0, im = 0;
           for (int64_t kk = lane; kk < nk; kk += 32) {
-            const int64_t ia = oa + map_offset(st.ka, kk), ib = ob + map_offset(st.kb, kk);
-            const double ar = A[ia], ai = A[st.pa + ia], br = B[ib], bi = B[st.pb + ib];
-            re += ar * br - ai * bi;
-            im += ar * bi + ai * br;
+            const int64_t ia = ka(kk), ib = kb(kk);
+            const double ar = Ao[ia], ai = Ao[st.pa + ia], br = Bo[ib], bi = Bo[st.pb + ib];
+            re = fma(-ai, bi, fma(ar, br, re));
+            im = fma(ai, br, fma(ar, bi, im));
           }
           for (int w = 16; w > 0; w >>= 1) {
             re += __shfl_xor_sync(0xffffffffu, re, w);
@@ -298,7 +328,7 @@ __global__ void __launch_bounds__(256) k_persistent(const InterpJob* __restrict_
           }
         }
       }
-      base += nout;
+      first += total;
     }
     __syncthreads();
   }
