@@ -60,6 +60,7 @@ using namespace dg;
 // ------------------------------------------------------------------ operand gathers
 
 constexpr int kTileElems = 2048;  // complex elements of a gather tile (at most)
+constexpr int kDigThreads = 512;  // gather threads: 256 units of 8 elements per plane
 
 // The exponent field (FP64 encoding) of a source value; zero and subnormal values give 0.
 __device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
@@ -83,13 +84,17 @@ struct TileMap {
   int nq;
   bool active;
 };
-__device__ __forceinline__ TileMap tile_map(const PermDev& p) {
+__device__ __forceinline__ TileMap tile_map(const PermDev& p, int tid) {
   TileMap t{0, 0, 1, true};
-  const int nb = p.tr + p.tk, tid = threadIdx.x;
-  for (int j = 0; j < 8 && j < nb; ++j)
-    if ((tid >> j) & 1) {
-      t.off += int64_t(1) << p.tsrc[j];
-      t.loc |= 1 << p.tloc[j];
+  const int nb = p.tr + p.tk;
+  const uint32_t* ws = reinterpret_cast<const uint32_t*>(p.tsrc);
+  const uint32_t* wl = reinterpret_cast<const uint32_t*>(p.tloc);
+  const uint32_t src[2] = {ws[0], ws[1]}, loc[2] = {wl[0], wl[1]};
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (j < nb && ((tid >> j) & 1)) {
+      t.off += int64_t(1) << ((src[j >> 2] >> (8 * (j & 3))) & 63);
+      t.loc |= 1 << ((loc[j >> 2] >> (8 * (j & 3))) & 15);
     }
   t.active = nb >= 8 || tid < (1 << nb);
   t.nq = nb > 8 ? 1 << (nb - 8) : 1;
@@ -129,7 +134,7 @@ __device__ __forceinline__ void row_exp_body(const PermDev& p, const S* __restri
   const int64_t R = int64_t(1) << p.rbits;
   const int TR = 1 << p.tr;
   const int64_t ntr = R >> p.tr, ntk = int64_t(1) << (p.kbits - p.tk), per = ntk / p.strips;
-  const TileMap tm = tile_map(p);
+  const TileMap tm = tile_map(p, threadIdx.x);
   const GroupMap gm(p);
   int* out = reinterpret_cast<int*>(base + p.dst[2]);
   for (int64_t it = blockIdx.x; it < ntr * p.strips; it += gridDim.x) {
@@ -203,91 +208,44 @@ __device__ __forceinline__ uint4 neg_f16x8(uint4 v) {
 // per real operand element. All arithmetic is on the integer and fp16 pipes (an FP64 instruction
 // per value would cost 32 times an integer one on GB300). Tiles of up to 2048 complex elements are
 // staged in shared memory: loads follow the source order, whatever it is, and stores write whole
-// 128-byte rows of the operand tiles, 16 bytes per thread.
+// 128-byte rows of the operand tiles, 16 bytes per thread. A thread has one plane's 8 values: with both
+// planes in one thread a block's chain of some 1,000 instructions per tile took 24 us even alone.
 template <typename S, int T>
 __device__ __forceinline__ void digits_body(const PermDev& p, const S* __restrict__ src, char* __restrict__ base,
                                             int64_t* tab, S* tre, S* tim) {
   const int c_r = nchunks(p.rows.nbits), c_k = nchunks(p.cols.nbits);
   int64_t* t_r = tab;
   int64_t* t_k = tab + c_r * 256;
-  build_table(p.rows, t_r);
-  build_table(p.cols, t_k);
-  chain_wait();
-  __syncthreads();
+  build_table<kDigThreads>(p.rows, t_r);
+  build_table<kDigThreads>(p.cols, t_k);
   const int64_t R = int64_t(1) << p.rbits, K = int64_t(1) << p.kbits;
   const int kt_bits = p.kbits - p.tk;              // log2 of the tiles along K
   const int64_t ntiles = int64_t(1) << (p.rbits - p.tr + kt_bits);
   const int ob = p.rbits + (p.embed ? 1 : 0);      // log2 of the operand's rows
-  const TileMap tm = tile_map(p);
+  const int plane = threadIdx.x >> 8, u = threadIdx.x & 255;  // unit: 8 consecutive local elements of one plane
+  const TileMap tm = tile_map(p, u);
   const GroupMap gm(p);
   const int ph = tile_place(tm.loc);
   char* dst = base + p.dst[0];
   int* exps = reinterpret_cast<int*>(base + p.dst[1]);
   const int* part = reinterpret_cast<const int*>(base + p.dst[2]);
-  const int u = threadIdx.x;                       // unit: 8 consecutive local elements
+  S* const mine = plane ? tim : tre;
   const bool unit = u < (1 << (p.tr + p.tk - 3));
   const int urow = (u << 3) >> p.tk, uk = (u << 3) & ((1 << p.tk) - 1);
   const int lanes = 1 << (p.tk - 3);               // units of one row of the tile
-  // digits of the unit's 8 values of a plane to row / column (r0, c0) and, negated or not, (r1, c1)
-  auto emit = [&](const S* plane, int E, int64_t r0, int64_t c0, bool two, int64_t r1, int64_t c1, bool neg) {
-    const Piece p0(ob, p.kbits + 1, T, r0, c0), p1(ob, p.kbits + 1, T, r1, c1);
-    int64_t y[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) y[j] = biased_fixed(f64_bits(plane[tile_place((u << 3) | j)]), E, T);
-#pragma unroll
-    for (int t = 0; t < T; ++t) {
-      uint32_t w[4];
-      if (t == T - 1) {
-        // the last digit with the rest: 18 bits, value (v - 2^17) 2^-9
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float f[2];
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const int v = static_cast<int>(static_cast<uint64_t>(y[2 * j + e]) >> (54 - 9 * t - 9)) & 0x3FFFF;
-            f[e] = static_cast<float>(v - 0x20000) * (1.0f / 512.0f);
-          }
-          const __half2 h = __floats2half2_rn(f[0], f[1]);
-          w[j] = *reinterpret_cast<const uint32_t*>(&h);
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint32_t f[2];
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            if (t == 0) f[e] = static_cast<uint32_t>(static_cast<int>(y[2 * j + e] >> 54) + 256);
-            else f[e] = static_cast<uint32_t>(static_cast<uint64_t>(y[2 * j + e]) >> (54 - 9 * t)) & 511u;
-          }
-          w[j] = pack_digits(f[0], f[1]);
-        }
-      }
-      const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
-      *reinterpret_cast<uint4*>(dst + p0.at(t)) = v;
-      if (two) *reinterpret_cast<uint4*>(dst + p1.at(t)) = neg ? neg_f16x8(v) : v;
-    }
-  };
+  chain_wait();
+  __syncthreads();
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t r0 = (tile >> kt_bits) << p.tr, k0 = (tile & ((int64_t(1) << kt_bits) - 1)) << p.tk;
     if (tm.active) {
-      const S* s0 = src + lookup(t_r, c_r, r0) + lookup(t_k, c_k, k0) + tm.off;
-      const S* s1 = s0 + p.plane;
-      S vr[8], vi[8];
+      const S* s0 = src + lookup(t_r, c_r, r0) + lookup(t_k, c_k, k0) + tm.off + (plane ? p.plane : 0);
+      S v[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (q < tm.nq) {
-          vr[q] = s0[gm.offset(q)];
-          vi[q] = s1[gm.offset(q)];
-        }
-      }
+      for (int q = 0; q < 8; ++q)
+        if (q < tm.nq) v[q] = s0[gm.offset(q)];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (q < tm.nq) {
-          const int at = ph ^ tile_place(gm.index(q));
-          tre[at] = vr[q];
-          tim[at] = vi[q];
-        }
-      }
+      for (int q = 0; q < 8; ++q)
+        if (q < tm.nq) mine[ph ^ tile_place(gm.index(q))] = v[q];
     }
     __syncthreads();
     if (unit) {
@@ -304,13 +262,45 @@ __device__ __forceinline__ void digits_body(const PermDev& p, const S* __restric
       } else {
         for (int s = 0; s < p.strips; ++s) E = max(E, part[s * R + r]);
       }
-      if (k == 0) exps[r] = E;
-      if (p.embed) {
-        emit(tre, E, r, k, true, R + r, K + k, false);   // Re at (s=0, t=0) and (s=1, t=1)
-        emit(tim, E, R + r, k, true, r, K + k, true);    // Im at (s=1, t=0), -Im at (s=0, t=1)
-      } else {
-        emit(tre, E, r, k, false, 0, 0, false);
-        emit(tim, E, r, K + k, false, 0, 0, false);
+      if (k == 0 && plane == 0) exps[r] = E;
+      int64_t y[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) y[j] = biased_fixed(f64_bits(mine[tile_place((u << 3) | j)]), E, T);
+      // embedded: Re at (s=0, t=0) and (s=1, t=1), Im at (s=1, t=0) and -Im at (s=0, t=1); plain: the
+      // plane's columns
+      const Piece p0(ob, p.kbits + 1, T, plane && p.embed ? R + r : r, plane && !p.embed ? K + k : k);
+      const Piece p1(ob, p.kbits + 1, T, plane ? r : R + r, K + k);
+#pragma unroll
+      for (int t = 0; t < T; ++t) {
+        uint32_t w[4];
+        if (t == T - 1) {
+          // the last digit with the rest: 18 bits, value (v - 2^17) 2^-9
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            float f[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const int v = static_cast<int>(static_cast<uint64_t>(y[2 * j + e]) >> (54 - 9 * t - 9)) & 0x3FFFF;
+              f[e] = static_cast<float>(v - 0x20000) * (1.0f / 512.0f);
+            }
+            const __half2 h = __floats2half2_rn(f[0], f[1]);
+            w[j] = *reinterpret_cast<const uint32_t*>(&h);
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            uint32_t f[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              if (t == 0) f[e] = static_cast<uint32_t>(static_cast<int>(y[2 * j + e] >> 54) + 256);
+              else f[e] = static_cast<uint32_t>(static_cast<uint64_t>(y[2 * j + e]) >> (54 - 9 * t)) & 511u;
+            }
+            w[j] = pack_digits(f[0], f[1]);
+          }
+        }
+        const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(dst + p0.at(t)) = v;
+        if (p.embed) *reinterpret_cast<uint4*>(dst + p1.at(t)) = plane ? neg_f16x8(v) : v;
       }
     }
     __syncthreads();
@@ -318,9 +308,9 @@ __device__ __forceinline__ void digits_body(const PermDev& p, const S* __restric
 }
 
 template <int T>
-__global__ void __launch_bounds__(kBodyThreads, 3) k_digits(const PermDev* __restrict__ perms,
-                                                            const double* __restrict__ arena, char* __restrict__ base,
-                                                            bool early) {
+__global__ void __launch_bounds__(kDigThreads, 2) k_digits(const PermDev* __restrict__ perms,
+                                                           const double* __restrict__ arena, char* __restrict__ base,
+                                                           bool early) {
   chain_trigger(early);
   extern __shared__ int64_t tab[];
   __shared__ __align__(16) double tile[2 * kTileElems];
@@ -875,7 +865,7 @@ cudaError_t launch_row_exp(const PermDev* d_perms, int nperm, int grid_x, size_t
 
 cudaError_t launch_digits(const PermDev* d_perms, int nperm, int grid_x, size_t smem, const void* arena, void* base,
                           int mode, cudaStream_t s, bool early) {
-  return launch_chained(mode == OPM_DIG6 ? k_digits<6> : k_digits<4>, dim3(grid_x, nperm), kBodyThreads, smem, s, d_perms,
+  return launch_chained(mode == OPM_DIG6 ? k_digits<6> : k_digits<4>, dim3(grid_x, nperm), kDigThreads, smem, s, d_perms,
                         static_cast<const double*>(arena), static_cast<char*>(base), early);
 }
 
