@@ -401,43 +401,9 @@ __device__ __forceinline__ float fixed_to_f32(int64_t acc, int e) {
   return __uint_as_float(s | ((static_cast<uint32_t>(f - 1) << 23) + m));
 }
 
-__device__ __forceinline__ bool elect_one() {
-  uint32_t ok;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
-  return ok != 0;
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(taddr));
-}
-template <int N>
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t* r) {
-  if constexpr (N == 16) tc::tmem_ld16(taddr, r);
-  else tmem_ld8(taddr, r);
-}
-
 // acc += v * mul, and acc += (v * mul) 2^32: one multiply-add each
 __device__ __forceinline__ void mad_wide(int64_t& acc, int v, int mul) { asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(v), "r"(mul)); }
 __device__ __forceinline__ void mad_high(int64_t& acc, int v, int mul) { acc += static_cast<int64_t>(static_cast<uint64_t>(static_cast<uint32_t>(v * mul)) << 32); }
-
-// One fp16 MMA (M = 128, K = 16) on operands given by the low words of their descriptors.
-template <bool kAcc>
-__device__ __forceinline__ void mma_f16(uint32_t tmem, uint32_t alo, uint32_t blo, uint32_t dhi, uint32_t idesc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
-      "mov.b64 a, {%1, %3};\n\t"
-      "mov.b64 b, {%2, %3};\n\t"
-      "setp.ne.b32 p, %5, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}" ::"r"(tmem),
-      "r"(alo), "r"(blo), "r"(dhi), "r"(idesc), "n"(kAcc ? 1 : 0)
-      : "memory");
-}
 
 template <int BC, int T, int PACK, typename Out>
 __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__ DgParams p) {
@@ -549,7 +515,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
 #pragma unroll
           for (int j0 = 0; j0 < COLS; j0 += CH) {
             uint32_t r[CH];
-            tmem_ld<CH>(t + j0, r);
+            tc::tmem_ld<CH>(t + j0, r);
             tc::tmem_wait_ld();
 #pragma unroll
             for (int j = 0; j < CH; ++j) mad_wide(acc[j0 + j], __float2int_rn(__uint_as_float(r[j]) * fs), 1);
@@ -567,7 +533,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
 #pragma unroll
           for (int j0 = 0; j0 < COLS; j0 += CH) {
             uint32_t r[CH];
-            tmem_ld<CH>(t + j0, r);
+            tc::tmem_ld<CH>(t + j0, r);
             tc::tmem_wait_ld();
 #pragma unroll
             for (int j = 0; j < CH; ++j) mad_wide(acc[j0 + j], __float2int_rn(__uint_as_float(r[j])), mul);
@@ -585,7 +551,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
 #pragma unroll
           for (int j0 = 0; j0 < COLS; j0 += CH) {
             uint32_t r[CH];
-            tmem_ld<CH>(t + j0, r);
+            tc::tmem_ld<CH>(t + j0, r);
             tc::tmem_wait_ld();
 #pragma unroll
             for (int j = 0; j < CH; ++j) mad_high(acc[j0 + j], __float2int_rn(__uint_as_float(r[j])), mul);
@@ -625,7 +591,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
     asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
   if (warp == 0) {
     // ---- producer: a chunk's slots, highest digits first (one lane issues)
-    const bool leader = elect_one();
+    const bool leader = tc::elect_one();
     const uint32_t ybytes = static_cast<uint32_t>(p.yrows) * 128u;
     int slot = 0;
     uint32_t phase = 0, issued = 0;
@@ -666,7 +632,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
     // per digit (the low words; the high word is constant), and the whole warp runs the loop with
     // values that the compiler can see are uniform. (Run by a single lane of a diverged warp, each MMA
     // cost 120 to 220 clocks of issue, and the kernel took 1.9 to 3.0 ms on 1024 x 32768 x 1024.)
-    const bool leader = elect_one();
+    const bool leader = tc::elect_one();
     int first = 0, buf = 0;
     uint32_t phase = 0, bphase = 0;
     bool any = false;
@@ -712,8 +678,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
               if (kk == 0 || kk < steps) {
-                if (fresh && kk == 0) mma_f16<false>(dst, y, x, dhi, p.idesc);
-                else mma_f16<true>(dst, y + 2 * kk, x + 2 * kk, dhi, p.idesc);
+                if (fresh && kk == 0) tc::mma<2, false>(dst, y, x, dhi, p.idesc);
+                else tc::mma<2, true>(dst, y + 2 * kk, x + 2 * kk, dhi, p.idesc);
               }
             }
             fresh = false;

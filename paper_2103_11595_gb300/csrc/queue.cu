@@ -53,9 +53,12 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 template <int BN, int KIND>
 __device__ __noinline__ bool gemm_task(const QPhase& ph, const QTask& t, const TcShared& sh, TcRing& ring) {
   const TcParams& p = *static_cast<const TcParams*>(ph.gemm);
-  if (threadIdx.x == 0) {
-    // the tensor maps live in global memory (written before the launch): acquire them for the
-    // tensor-map proxy before the producer's first TMA load through them
+  if (threadIdx.x < 32) {
+    // the producer warp, whichever lane issues its copies: the operands were written by other blocks
+    // through the generic proxy, and the tensor maps live in global memory (written before the launch):
+    // acquire them for the tensor-map proxy before the first TMA load through them
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     for (int i = 0; i < p.terms; ++i) {
       asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&p.amap[i]) : "memory");
       asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&p.bmap[i]) : "memory");

@@ -67,7 +67,7 @@ namespace {
 
 using namespace tc;
 
-template <int BN, int kKind>
+template <int BN, int kKind, int kT>
 __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__ TcParams p, bool early) {
   chain_trigger(early);
   extern __shared__ uint8_t smem_raw[];
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
   chain_wait();
   TcRing ring;
   const uint32_t nwork = static_cast<uint32_t>(p.tiles) * static_cast<uint32_t>(p.ksplit);
-  tc_gemm_items<BN, kKind>(p, blockIdx.x, nwork, gridDim.x, sh, ring);
+  tc_gemm_terms<BN, kKind, kT>(p, blockIdx.x, nwork, gridDim.x, sh, ring);
   if (*sh.abort_flag) tc_drain_after_abort(p.slots, p.bufs, p.wait_ns, p.status, sh, ring);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   // __syncthreads (bar.sync, the aligned form) must be executed by all threads of a warp
@@ -147,14 +147,14 @@ int sm_count() {
   return counts[dev];
 }
 
-template <int BN, int KIND>
+template <int BN, int KIND, int T>
 cudaError_t run_tile(const void* params, unsigned grid, size_t smem, cudaStream_t s, bool early) {
-  return launch_chained(k_gemm_tc<BN, KIND>, dim3(grid), kThreads, smem, s, *static_cast<const TcParams*>(params), early);
+  return launch_chained(k_gemm_tc<BN, KIND, T>, dim3(grid), kThreads, smem, s, *static_cast<const TcParams*>(params), early);
 }
 
 // Fill the tile geometry of `p` and the launch shape of `t` (host only; nothing is enqueued).
-template <int BN, int KIND>
-cudaError_t prepare_tile(TcParams& p, TcPrepared* t, int64_t M, int64_t N) {
+template <int BN, int KIND, int T>
+cudaError_t prepare_terms(TcParams& p, TcPrepared* t, int64_t M, int64_t N) {
   p.slot_bytes = static_cast<uint32_t>((kBM + BN) * kRowBytes);
   p.slots = static_cast<int32_t>(kSmemBudget / p.slot_bytes);
   if (p.slots > kMaxSlots) p.slots = kMaxSlots;
@@ -190,14 +190,21 @@ cudaError_t prepare_tile(TcParams& p, TcPrepared* t, int64_t M, int64_t N) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    e = cudaFuncSetAttribute(k_gemm_tc<BN, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    e = cudaFuncSetAttribute(k_gemm_tc<BN, KIND, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) attr_set[dev] = true;
   }
   t->grid = static_cast<unsigned>(grid);
   t->smem = smem;
-  t->run = &run_tile<BN, KIND>;
+  t->run = &run_tile<BN, KIND, T>;
   return cudaSuccess;
+}
+
+template <int BN, int KIND>
+cudaError_t prepare_tile(TcParams& p, TcPrepared* t, int64_t M, int64_t N) {
+  if (KIND != 2 && p.terms == 1) return prepare_terms<BN, KIND, 1>(p, t, M, N);
+  if (KIND != 2 && p.terms == 3) return prepare_terms<BN, KIND, 3>(p, t, M, N);
+  return prepare_terms<BN, KIND, 2>(p, t, M, N);
 }
 
 }  // namespace

@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "kernels.h"
 
@@ -127,23 +128,35 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
   return d;
 }
 
+// One lane of the (converged) warp, the same one every time.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok));
+  return ok != 0;
+}
+
 // Operand kinds: 0 TF32 (kind::tf32), 1 bf16, 2 fp16 scaled per row and K block (kind::f16; the
-// instruction descriptor names the type).
-template <int kKind>
-__device__ __forceinline__ void mma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+// instruction descriptor names the type). The operands are given by the low words of their
+// descriptors and the common high word.
+template <int kKind, bool kAcc>
+__device__ __forceinline__ void mma(uint32_t tmem, uint32_t alo, uint32_t blo, uint32_t dhi, uint32_t idesc) {
   if (kKind != 0) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+        "mov.b64 a, {%1, %3};\n\t"
+        "mov.b64 b, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}" ::"r"(tmem),
+        "r"(alo), "r"(blo), "r"(dhi), "r"(idesc), "n"(kAcc ? 1 : 0)
         : "memory");
   } else {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+        "mov.b64 a, {%1, %3};\n\t"
+        "mov.b64 b, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], a, b, %4, p;\n\t}" ::"r"(tmem),
+        "r"(alo), "r"(blo), "r"(dhi), "r"(idesc), "n"(kAcc ? 1 : 0)
         : "memory");
   }
 }
@@ -159,6 +172,17 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+template <int N>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t* r) {
+  if constexpr (N == 16) tmem_ld16(taddr, r);
+  else tmem_ld8(taddr, r);
 }
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -241,20 +265,31 @@ __device__ __forceinline__ void tc_init_barriers(const TcShared& sh, int S, int 
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// Work items wi0, wi0 + step, ... (< wi1) of one GEMM, run by the block's three roles: warp 0
-// lane 0 the TMA producer, warp 1 lane 0 the MMA issuer, warps 2..9 the epilogue; the other
-// lanes of warps 0 and 1 pass straight through. Returns false in a role that gave up (a bounded
-// wait expired, or another role set the abort flag); the roles' ring positions advance in `r`.
-template <int BN, int kKind>
-__device__ __forceinline__ bool tc_gemm_items(const TcParams& p, uint32_t wi0, uint32_t wi1, uint32_t step,
+// Work items wi0, wi0 + step, ... (< wi1) of one GEMM of kT split terms, run by the block's three roles:
+// warp 0 the TMA producer, warp 1 the MMA issuer, warps 2..9 the epilogue. Returns false in a role that
+// gave up (a bounded wait expired, or another role set the abort flag); the roles' ring positions
+// advance in `r`. All threads of the block call it, the lanes of a warp together.
+// At N = 128 the issue of the MMAs (64 clocks each) is what bounds long products: with one lane of a
+// diverged warp running the issuer's loop 1024 x 32768 x 1024 (bf16x6) took 328 us, with the whole warp
+// on uniform values, an elected lane and unrolled products 308 us (1,340 TFLOP/s of bf16 products);
+// without loads or epilogue arithmetic, the same.
+template <int BN, int kKind, int kT>
+__device__ __forceinline__ bool tc_gemm_terms(const TcParams& p, uint32_t wi0, uint32_t wi1, uint32_t step,
                                               const TcShared& sh, TcRing& r) {
   static_assert(BN == 32 || BN == 64 || BN == 128, "tile width");
   constexpr int COLS = BN / 2;                       // columns per epilogue thread (one TMEM lane = one row)
-  constexpr int CH = COLS < 16 ? COLS : 16;          // columns per drain chunk
+  constexpr int CH = kT > 1 ? 8 : 16;                // columns per drain chunk (two partials: no spills)
   constexpr uint32_t a_bytes = kBM * kRowBytes, b_bytes = BN * kRowBytes;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int S = p.slots, T = p.terms, NB = p.bufs;
-  const uint32_t tmem = sh.tmem;
+  // The producer's and issuer's values are the same in every lane of their warps and, through these
+  // shuffles and the votes on waits, known to be: addresses and descriptors then live in uniform
+  // registers, where the copy and tensor instructions take them from, and one elected lane issues.
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const int S = p.slots, NB = p.bufs;
+  constexpr int T = kT;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, sh.tmem, 0);
+  auto warp_wait = [&](uint32_t bar, uint32_t parity, int code) {
+    return __all_sync(0xffffffffu, !*sh.abort_flag && mbar_wait(bar, parity, p.wait_ns, p.status, code)) != 0;
+  };
   // persistent tile loop: every role walks the same work items, and its ring positions (slots,
   // TMEM buffers) continue across items. Grouped raster: `group` M tiles sweep the N tiles
   // together, so concurrently running CTAs share each B tile through L2 instead of streaming all
@@ -273,29 +308,29 @@ __device__ __forceinline__ bool tc_gemm_items(const TcParams& p, uint32_t wi0, u
     kb1 = kb0 + p.kb_split < p.kblocks ? kb0 + p.kb_split : p.kblocks;
   };
   bool ok = true;
-  if (warp == 0 && lane == 0) {
-    // ---- TMA producer: one slot per (K block, term) holds that term's A and B tiles. A block's
-    // terms are loaded highest first, the order in which the MMA issuer frees their slots.
-    int slot = r.slot;
-    uint32_t phase = r.phase, issued = r.issued;
+  if (warp == 0) {
+    // ---- TMA producer: one slot per (K block, term) holds that term's A and B tiles. A block's terms
+    // are loaded highest first, the order in which the MMA issuer frees their slots.
+    const bool leader = elect_one();
+    int slot = __shfl_sync(0xffffffffu, r.slot, 0);
+    uint32_t phase = __shfl_sync(0xffffffffu, r.phase, 0), issued = r.issued;
     ok = !p.stall_loads;
     for (uint32_t wi = wi0; wi < wi1 && ok; wi += step) {
       int32_t m0, n0;
       int kb0, kb1;
       work_item(wi, m0, n0, kb0, kb1);
       for (int kb = kb0; kb < kb1 && ok; ++kb) {
-        for (int j = 0; j < T; ++j) {
-          const int t = T - 1 - j;
-          if (*sh.abort_flag || !mbar_wait(sh.empty0 + 8 * slot, phase ^ 1u, p.wait_ns, p.status, 11)) {
-            *sh.abort_flag = 1;
-            ok = false;
-            break;
+        const int32_t kx = kb * (kRowBytes / (kKind != 0 ? 2 : 4));
+#pragma unroll 1
+        for (int t = T - 1; t >= 0; --t) {
+          ok = warp_wait(sh.empty0 + 8 * slot, phase ^ 1u, 11);
+          if (!ok) break;
+          const uint32_t sa = smem_u32(sh.slots + slot * p.slot_bytes), bar = sh.full0 + 8 * slot;
+          if (leader) {
+            mbar_expect_tx(bar, a_bytes + b_bytes);
+            tma_load_2d(sa, &p.amap[t], kx, m0, bar);
+            tma_load_2d(sa + a_bytes, &p.bmap[t], kx, n0, bar);
           }
-          const uint32_t sa = smem_u32(sh.slots + slot * p.slot_bytes);
-          const int32_t kx = kb * (kRowBytes / (kKind != 0 ? 2 : 4));
-          mbar_expect_tx(sh.full0 + 8 * slot, a_bytes + b_bytes);
-          tma_load_2d(sa, &p.amap[t], kx, m0, sh.full0 + 8 * slot);
-          tma_load_2d(sa + a_bytes, &p.bmap[t], kx, n0, sh.full0 + 8 * slot);
           ++issued;
           if (++slot == S) {
             slot = 0;
@@ -304,111 +339,96 @@ __device__ __forceinline__ bool tc_gemm_items(const TcParams& p, uint32_t wi0, u
         }
       }
     }
+    if (!ok && lane == 0) *sh.abort_flag = 1;
     r.slot = slot;
     r.phase = phase;
     r.issued = issued;
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---- MMA issuer
-    int buf = r.mbuf, slot = r.mslot;
-    uint32_t bphase = r.mbphase, phase = r.mphase;
+    const bool leader = elect_one();
+    int buf = __shfl_sync(0xffffffffu, r.mbuf, 0), slot = __shfl_sync(0xffffffffu, r.mslot, 0);
+    uint32_t bphase = __shfl_sync(0xffffffffu, r.mbphase, 0), phase = __shfl_sync(0xffffffffu, r.mphase, 0);
+    const uint64_t desc0 = smem_desc(smem_u32(sh.slots));
+    const uint32_t dlo0 = static_cast<uint32_t>(desc0), dhi = static_cast<uint32_t>(desc0 >> 32);
     for (uint32_t wi = wi0; wi < wi1 && ok; wi += step) {
       int32_t m0, n0;
       int kb0, kb1;
       work_item(wi, m0, n0, kb0, kb1);
       for (int kb = kb0; kb < kb1; ++kb) {
         const int b = buf;
-        if (*sh.abort_flag || !mbar_wait(sh.acce0 + 8 * b, bphase ^ 1u, p.wait_ns, p.status, 14)) {
-          ok = false;
-          break;
-        }
+        ok = warp_wait(sh.acce0 + 8 * b, bphase ^ 1u, 14);
+        if (!ok) break;
         if (kKind == 2) {
           // the K block's row and column scales into buffer b's scale area (the epilogue has
           // released the buffer, so also its scales)
           const uint32_t rows = static_cast<uint32_t>(p.M - m0 < kBM ? p.M - m0 : kBM);
           const uint32_t cols = static_cast<uint32_t>(p.N - n0 < BN ? p.N - n0 : BN);
           const uint32_t sdst = smem_u32(sh.scales + b * kScaleFloats);
-          mbar_expect_tx(sh.sfull0 + 8 * b, 4 * (rows + cols));
-          bulk_load(sdst, p.sa + static_cast<int64_t>(kb) * p.M + m0, 4 * rows, sh.sfull0 + 8 * b);
-          bulk_load(sdst + 4 * 128, p.sb + static_cast<int64_t>(kb) * p.N + n0, 4 * cols, sh.sfull0 + 8 * b);
+          if (leader) {
+            mbar_expect_tx(sh.sfull0 + 8 * b, 4 * (rows + cols));
+            bulk_load(sdst, p.sa + static_cast<int64_t>(kb) * p.M + m0, 4 * rows, sh.sfull0 + 8 * b);
+            bulk_load(sdst + 4 * 128, p.sb + static_cast<int64_t>(kb) * p.N + n0, 4 * cols, sh.sfull0 + 8 * b);
+          }
           ++r.scopies;
         }
         if (++buf == NB) {
           buf = 0;
           bphase ^= 1u;
         }
-        // ring positions of the block's slots (the producer loads term T-1 first), then the slot
-        // and phase of each term; all in scalars -- descriptors and slots kept in registers (a
-        // dynamically indexed array would live in local memory and stall every MMA issue)
-        int r0 = slot, r1 = 0, r2 = 0;
-        uint32_t f0 = phase, f1 = 0u, f2 = 0u;
-        auto advance = [&]() {
+        // slot and phase of each term (the producer loads term T - 1 first)
+        int st[T];
+        uint32_t ph[T];
+#pragma unroll
+        for (int t = T - 1; t >= 0; --t) {
+          st[t] = slot;
+          ph[t] = phase;
           if (++slot == S) {
             slot = 0;
             phase ^= 1u;
           }
-        };
-        advance();
-        if (T > 1) {
-          r1 = slot;
-          f1 = phase;
-          advance();
         }
-        if (T > 2) {
-          r2 = slot;
-          f2 = phase;
-          advance();
-        }
-        const int st0 = T == 3 ? r2 : (T == 2 ? r1 : r0), st1 = T == 3 ? r1 : r0, st2 = r0;
-        const uint32_t ph0 = T == 3 ? f2 : (T == 2 ? f1 : f0), ph1 = T == 3 ? f1 : f0, ph2 = f0;
-        const uint32_t base = smem_u32(sh.slots);
-        const uint64_t ad0 = smem_desc(base + st0 * p.slot_bytes), bd0 = smem_desc(base + st0 * p.slot_bytes + a_bytes);
-        const uint64_t ad1 = smem_desc(base + st1 * p.slot_bytes), bd1 = smem_desc(base + st1 * p.slot_bytes + a_bytes);
-        const uint64_t ad2 = smem_desc(base + st2 * p.slot_bytes), bd2 = smem_desc(base + st2 * p.slot_bytes + a_bytes);
         const uint32_t dst0 = tmem + static_cast<uint32_t>(b * p.tmem_stride);  // P0: the leading product alone
         const uint32_t dst1 = dst0 + static_cast<uint32_t>(BN);                 // P1: the correction products
-        uint32_t acc = 0;
         // one product A_i . B_j over the block: 4 instructions, 32 bytes of K each (+2 in the
-        // descriptor's 16-byte address field)
-        auto product = [&](uint32_t dst, uint64_t ad, uint64_t bd) {
+        // descriptor's 16-byte address field); a term's B tile follows its A tile
+        auto product = [&](uint32_t dst, int i, int j, auto fresh) {
+          const uint32_t a = dlo0 + st[i] * (p.slot_bytes >> 4), bb = dlo0 + st[j] * (p.slot_bytes >> 4) + (a_bytes >> 4);
+          mma<kKind, !decltype(fresh)::value>(dst, a, bb, dhi, p.idesc);
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            mma<kKind>(dst, ad + 2 * kk, bd + 2 * kk, p.idesc, acc);
-            acc = 1;
-          }
+          for (int kk = 1; kk < 4; ++kk) mma<kKind, true>(dst, a + 2 * kk, bb + 2 * kk, dhi, p.idesc);
         };
-        auto arrived = [&](int sl, uint32_t ph) {
-          const bool w = mbar_wait(sh.full0 + 8 * sl, ph, p.wait_ns, p.status, 12);
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          return w;
-        };
+        using First = std::true_type;
+        using Next = std::false_type;
         // all of the block's terms are resident before its first MMA (a failed wait then leaves
         // nothing of this block in flight); the correction products go into P1 smallest first, the
         // leading product into P0, and a term's slot is released (commit: freed once the MMAs
         // issued so far complete) right after its last use
-        const bool got = (T < 3 || arrived(st2, ph2)) && (T < 2 || arrived(st1, ph1)) && arrived(st0, ph0);
-        if (!got) {
-          ok = false;
-          break;
-        }
+#pragma unroll
+        for (int t = T - 1; t >= 0; --t) ok = ok && warp_wait(sh.full0 + 8 * st[t], ph[t], 12);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (!ok) break;
         r.any = true;
-        if (T == 3) {
-          product(dst1, ad0, bd2);
-          product(dst1, ad1, bd1);
-          product(dst1, ad2, bd0);
-          mma_commit(sh.empty0 + 8 * st2);
+        if (leader) {
+          if constexpr (T == 3) {
+            product(dst1, 0, 2, First());
+            product(dst1, 1, 1, Next());
+            product(dst1, 2, 0, Next());
+            mma_commit(sh.empty0 + 8 * st[2]);
+            product(dst1, 0, 1, Next());
+            product(dst1, 1, 0, Next());
+            mma_commit(sh.empty0 + 8 * st[1]);
+          } else if constexpr (T == 2) {
+            product(dst1, 0, 1, First());
+            product(dst1, 1, 0, Next());
+            mma_commit(sh.empty0 + 8 * st[1]);
+          }
+          product(dst0, 0, 0, First());
+          mma_commit(sh.empty0 + 8 * st[0]);
+          mma_commit(sh.accf0 + 8 * b);
         }
-        if (T >= 2) {
-          product(dst1, ad0, bd1);
-          product(dst1, ad1, bd0);
-          mma_commit(sh.empty0 + 8 * st1);
-        }
-        acc = 0;
-        product(dst0, ad0, bd0);
-        mma_commit(sh.empty0 + 8 * st0);
-        mma_commit(sh.accf0 + 8 * b);
       }
     }
-    if (!ok) *sh.abort_flag = 1;
+    if (!ok && lane == 0) *sh.abort_flag = 1;
     r.mbuf = buf;
     r.mslot = slot;
     r.mbphase = bphase;
@@ -466,10 +486,10 @@ __device__ __forceinline__ bool tc_gemm_items(const TcParams& p, uint32_t wi0, u
         for (int c0 = 0; c0 < COLS; c0 += CH) {
           uint32_t r0[CH], r1[CH];
 #pragma unroll
-          for (int c1 = 0; c1 < CH; c1 += 16) tmem_ld16(tmem + lane_base + col + c0 + c1, r0 + c1);
+          for (int c1 = 0; c1 < CH; c1 += 16) tmem_ld<CH>(tmem + lane_base + col + c0 + c1, r0 + c1);
           if (T > 1) {
 #pragma unroll
-            for (int c1 = 0; c1 < CH; c1 += 16) tmem_ld16(tmem + lane_base + col + BN + c0 + c1, r1 + c1);
+            for (int c1 = 0; c1 < CH; c1 += 16) tmem_ld<CH>(tmem + lane_base + col + BN + c0 + c1, r1 + c1);
           }
           tmem_wait_ld();
           if (kKind == 2) {
@@ -534,6 +554,15 @@ __device__ __forceinline__ bool tc_gemm_items(const TcParams& p, uint32_t wi0, u
     r.ebphase = bphase;
   }
   return ok;
+}
+
+// The same for the number of split terms in `p` (the interpreter).
+template <int BN, int kKind>
+__device__ __forceinline__ bool tc_gemm_items(const TcParams& p, uint32_t wi0, uint32_t wi1, uint32_t step,
+                                              const TcShared& sh, TcRing& r) {
+  if (kKind != 2 && p.terms == 1) return tc_gemm_terms<BN, kKind, 1>(p, wi0, wi1, step, sh, r);
+  if (kKind != 2 && p.terms == 3) return tc_gemm_terms<BN, kKind, 3>(p, wi0, wi1, step, sh, r);
+  return tc_gemm_terms<BN, kKind, 2>(p, wi0, wi1, step, sh, r);
 }
 
 // After an abort (the abort flag set), before the block releases its shared memory and TMEM: the
