@@ -362,8 +362,9 @@ def main():
     pk = peaks()
     d = classes[dom]
     if dom == "gemm_tc":
-        passes = {"tf32": 1, "tf32x3": 3, "bf16x3": 3, "bf16x6": 6, "f16x3": 3}[args.precision]
-        if args.precision.startswith("bf16") or args.precision.startswith("f16"):
+        # hardware products per algorithmic one; the f64 and f32 modes' GEMMs are sums of fp16 digit products
+        passes = {"tf32": 1, "tf32x3": 3, "bf16x3": 3, "bf16x6": 6, "f16x3": 3, "f64": 26, "f32": 10}[args.precision]
+        if not args.precision.startswith("tf32"):
             peak = pk["bf16_tflops"]
             src = f"{pk['src']} bf16 dense burst (MEASURED_PEAKS.json)"
         else:
