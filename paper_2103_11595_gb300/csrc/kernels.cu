@@ -13,7 +13,8 @@
 //                with the operand format of the precision mode (FP64, FP32, TF32, split TF32,
 //                split bf16).
 //  k_gemm_simt   real "TN" GEMM on CUDA cores (FP32 or FP64) writing the planar result.
-//  k_open/k_final  the FP64 end of the path: t_i for Alg. I, sum |t_i|^2, F_J and 1 - F_J.
+//  k_open/k_final  the FP64 end of the path: t_i for Alg. I, sum |t_i|^2, F_J and 1 - F_J; k_open_final
+//                both, when one block covers the open tensor.
 #include <algorithm>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

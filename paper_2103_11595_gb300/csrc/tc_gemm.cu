@@ -34,10 +34,10 @@
 // Kernel structure (persistent: at most one CTA per SM walks the 128 x BN output tiles in a
 // grouped raster order; 320 threads; the slot and TMEM-buffer rings continue from tile to tile so
 // the loads and MMAs of the next tile overlap the store of the current one):
-//   warp 0, lane 0 : TMA producer -- for every K block and term, the A tile (128 rows x 128 B) and
+//   warp 0         : TMA producer (an elected lane issues) -- for every K block and term, the A tile (128 rows x 128 B) and
 //                    the B tile (BN rows x 128 B), 128-byte swizzle, into a ring of slots
 //                    (mbarrier expect-tx / complete-tx);
-//   warp 1         : allocates TMEM; lane 0 issues tcgen05.mma (M=128, N=BN, 32 B of K each) into
+//   warp 1         : allocates TMEM; an elected lane issues tcgen05.mma (M=128, N=BN, 32 B of K each) into
 //                    a ring of TMEM buffers (two partials of BN columns each) and tcgen05.commit
 //                    to release slots and hand partials to the epilogue;
 //   warps 2..9     : epilogue -- two warps per TMEM lane quarter (warp % 4), each owning half of
