@@ -44,6 +44,8 @@ struct SyncBody {  // threads 0..kBodyThreads-1 of a larger block: named barrier
 };
 
 // Chained launches (kernels.h, launch_chained): the successor may start / everything before is complete.
+// The bodies below run in such kernels, and as tasks of the interpreter beside the blocks that write their
+// operands: their pointers to tensors and partial sums are not __restrict__.
 __device__ __forceinline__ void chain_trigger(bool early) {
   if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
@@ -125,7 +127,7 @@ __device__ __forceinline__ void with_operands(const double* arena, int64_t a, bo
 // ------------------------------------------------------------------ leaves
 
 // Element e of leaf L (complex, FP64) from the uploaded complex128 matrices.
-__device__ __forceinline__ void leaf_value(const LeafDev& L, const double* __restrict__ in, int64_t e, double& re,
+__device__ __forceinline__ void leaf_value(const LeafDev& L, const double* in, int64_t e, double& re,
                                            double& im) {
   re = 0;
   im = 0;
@@ -186,7 +188,7 @@ __device__ __forceinline__ int64_t leaf_full_index(const LeafDev& L, int64_t e) 
 
 // One leaf per (virtual) block.
 template <typename T>
-__device__ __forceinline__ void leaf_body(const LeafDev* leaves, const double* __restrict__ in, T* __restrict__ arena,
+__device__ __forceinline__ void leaf_body(const LeafDev* leaves, const double* in, T* arena,
                                           int vb) {
   const LeafDev L = leaves[vb];
   const int64_t n = int64_t(1) << L.bits;
@@ -243,7 +245,7 @@ __device__ __forceinline__ double widen(float x) {
 // clocks.
 template <typename T, typename Acc, typename Sync, int kThreads = kBodyThreads>
 __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, int nsteps, int total_blocks,
-                                           T* __restrict__ arena, int vb, int64_t* tab, StepDev& st) {
+                                           T* arena, int vb, int64_t* tab, StepDev& st) {
   const int s = find_step(steps, nsteps, vb);
   const int end = (s + 1 < nsteps) ? steps[s + 1].block0 : total_blocks;
   static_assert(sizeof(StepDev) % 4 == 0, "descriptor copy");
@@ -322,8 +324,8 @@ __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, in
 
 
 template <typename T, typename Sync>
-__device__ __forceinline__ void splitk_body(const StepDev* __restrict__ steps, int nsteps, const T* __restrict__ arena,
-                                            double2* __restrict__ partial, int vb, int64_t* tab, double* red_re,
+__device__ __forceinline__ void splitk_body(const StepDev* __restrict__ steps, int nsteps, const T* arena,
+                                            double2* partial, int vb, int64_t* tab, double* red_re,
                                             double* red_im) {
   const int s = find_step(steps, nsteps, vb);
   const StepDev& st = steps[s];
@@ -396,8 +398,8 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 template <typename T, bool kF32, typename Sync, bool kStaged = false>
-__device__ __forceinline__ void dot_body(const StepDev* __restrict__ steps, int nsteps, const T* __restrict__ arena,
-                                         double2* __restrict__ partial, int vb, int64_t* tab, double* red_re,
+__device__ __forceinline__ void dot_body(const StepDev* __restrict__ steps, int nsteps, const T* arena,
+                                         double2* partial, int vb, int64_t* tab, double* red_re,
                                          double* red_im) {
   const int s = find_step(steps, nsteps, vb);
   const StepDev& st = steps[s];
@@ -666,8 +668,8 @@ __device__ __forceinline__ void dot_body(const StepDev* __restrict__ steps, int 
 // whole block reduces each output (strided per-thread sums, then a tree), otherwise one thread
 // sums one output's splits.
 template <typename T, typename Sync>
-__device__ __forceinline__ void splitk_done_body(const StepDev* __restrict__ steps, const double2* __restrict__ partial,
-                                                 T* __restrict__ arena, double2* __restrict__ scalars, int vb,
+__device__ __forceinline__ void splitk_done_body(const StepDev* __restrict__ steps, const double2* partial,
+                                                 T* arena, double2* scalars, int vb,
                                                  double* red_re, double* red_im) {
   const StepDev& st = steps[vb];
   const int64_t nout = int64_t(1) << st.rc;
@@ -856,8 +858,8 @@ __device__ __forceinline__ uint4 neg_bf16x8(uint4 v) {
 // second copies reuse the split (-Im is Im with the sign bits flipped). Two barriers per tile.
 // The values are those of the general loop below, which handles every other case.
 template <typename Sync>
-__device__ __forceinline__ void perm_tiles_bf16x3(const PermDev& p, const double* __restrict__ arena,
-                                                  char* __restrict__ base, int vb, int vg, const int64_t* t_r,
+__device__ __forceinline__ void perm_tiles_bf16x3(const PermDev& p, const double* arena,
+                                                  char* base, int vb, int vg, const int64_t* t_r,
                                                   int c_r, const int64_t* t_k, int c_k, PermSmem<float>& sm,
                                                   PermSmem<float>* sm2) {
   const int64_t R = int64_t(1) << p.rbits, K = int64_t(1) << p.kbits;
@@ -997,8 +999,8 @@ __device__ __forceinline__ void perm_tiles_bf16x3(const PermDev& p, const double
 }
 
 template <typename S, typename Sync>
-__device__ __forceinline__ void perm_body(const PermDev* __restrict__ perms, const double* __restrict__ arena,
-                                          char* __restrict__ base, int vb, int vg, int vy, int64_t* tab,
+__device__ __forceinline__ void perm_body(const PermDev* __restrict__ perms, const double* arena,
+                                          char* base, int vb, int vg, int vy, int64_t* tab,
                                           PermSmem<S>& sm, PermSmem<float>* sm2 = nullptr) {
   constexpr int TKMAX = PermSmem<S>::TKMAX;
   auto& tre = sm.tre;
@@ -1154,9 +1156,9 @@ __device__ __forceinline__ void perm_body(const PermDev* __restrict__ perms, con
 // ------------------------------------------------------------------ final FP64 reduction
 
 template <typename T, typename Sync>
-__device__ __forceinline__ void open_body(const FinalDev* __restrict__ fd, const T* __restrict__ arena,
-                                          const double2* __restrict__ scalars, double* __restrict__ traces,
-                                          double* __restrict__ partial, int vb, int vg, int64_t* tab, double* red) {
+__device__ __forceinline__ void open_body(const FinalDev* __restrict__ fd, const T* arena,
+                                          const double2* scalars, double* traces,
+                                          double* partial, int vb, int vg, int64_t* tab, double* red) {
   const FinalDev& f = *fd;
   // common factor: product of scalar components and 2 per untouched wire
   double sr = ldexp(1.0, f.loops), si = 0;
@@ -1199,8 +1201,8 @@ __device__ __forceinline__ void open_body(const FinalDev* __restrict__ fd, const
 }
 
 // Thread 0 only.
-__device__ __forceinline__ void final_body(const FinalDev* __restrict__ fd, const double2* __restrict__ scalars,
-                                           const double* __restrict__ partial, double* __restrict__ result) {
+__device__ __forceinline__ void final_body(const FinalDev* __restrict__ fd, const double2* scalars,
+                                           const double* partial, double* result) {
   const FinalDev& f = *fd;
   double S = 0;
   if (f.alg == 2) {
@@ -1225,8 +1227,8 @@ __device__ __forceinline__ void final_body(const FinalDev* __restrict__ fd, cons
 // tensor-core GEMM, added in FP32 with Kahan's compensation (the sum's error stays within a few
 // units in the last place of the largest partial, whatever the number of splits; no FP64
 // arithmetic, which GB300 runs at a small fraction of its FP32 rate).
-__device__ __forceinline__ void split_sum_body(const float* __restrict__ W, int ksplit, int64_t n,
-                                               float* __restrict__ C, int vb, int vg) {
+__device__ __forceinline__ void split_sum_body(const float* W, int ksplit, int64_t n,
+                                               float* C, int vb, int vg) {
   for (int64_t i = int64_t(vb) * kBodyThreads + threadIdx.x; i < n; i += int64_t(vg) * kBodyThreads) {
     float s = 0.0f, comp = 0.0f;
     for (int k = 0; k < ksplit; ++k) {

@@ -122,7 +122,7 @@ struct GroupMap {
 // Largest exponent field of every complex row over strips of its K (dst[2]: [strip][row]). Only
 // the exponents are needed: one pass of reads, bound by HBM.
 template <typename S>
-__device__ __forceinline__ void row_exp_body(const PermDev& p, const S* __restrict__ src, char* __restrict__ base,
+__device__ __forceinline__ void row_exp_body(const PermDev& p, const S* src, char* base,
                                              int64_t* tab, int* rmax) {
   const int c_r = nchunks(p.rows.nbits), c_k = nchunks(p.cols.nbits);
   int64_t* t_r = tab;
@@ -175,7 +175,7 @@ __device__ __forceinline__ void row_exp_body(const PermDev& p, const S* __restri
 }
 
 __global__ void __launch_bounds__(kBodyThreads, 4) k_row_exp(const PermDev* __restrict__ perms,
-                                                             const double* __restrict__ arena, char* __restrict__ base) {
+                                                             const double* arena, char* base) {
   extern __shared__ int64_t tab[];
   __shared__ int rmax[256];
   const PermDev& p = perms[blockIdx.y];
@@ -211,7 +211,7 @@ __device__ __forceinline__ uint4 neg_f16x8(uint4 v) {
 // 128-byte rows of the operand tiles, 16 bytes per thread. A thread has one plane's 8 values: with both
 // planes in one thread a block's chain of some 1,000 instructions per tile took 24 us even alone.
 template <typename S, int T>
-__device__ __forceinline__ void digits_body(const PermDev& p, const S* __restrict__ src, char* __restrict__ base,
+__device__ __forceinline__ void digits_body(const PermDev& p, const S* src, char* base,
                                             int64_t* tab, S* tre, S* tim) {
   const int c_r = nchunks(p.rows.nbits), c_k = nchunks(p.cols.nbits);
   int64_t* t_r = tab;
@@ -309,7 +309,7 @@ __device__ __forceinline__ void digits_body(const PermDev& p, const S* __restric
 
 template <int T>
 __global__ void __launch_bounds__(kDigThreads, 2) k_digits(const PermDev* __restrict__ perms,
-                                                           const double* __restrict__ arena, char* __restrict__ base,
+                                                           const double* arena, char* base,
                                                            bool early) {
   chain_trigger(early);
   extern __shared__ int64_t tab[];
@@ -728,8 +728,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
 
 // C[i] = sum over K splits (in order) of W[s][i]
 template <typename Out>
-__global__ void __launch_bounds__(kBodyThreads) k_dg_split_sum(const double* __restrict__ W, int ksplit, int64_t n,
-                                                               Out* __restrict__ C) {
+__global__ void __launch_bounds__(kBodyThreads) k_dg_split_sum(const double* W, int ksplit, int64_t n,
+                                                               Out* C) {
   chain_wait();
   for (int64_t i = int64_t(blockIdx.x) * kBodyThreads + threadIdx.x; i < n; i += int64_t(gridDim.x) * kBodyThreads) {
     double s = W[i];

@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(kBodyThreads) k_leaf(const LeafDev* leaves, co
 
 template <typename T, typename Acc>
 __global__ void __launch_bounds__(kSmallThreads) k_small(const StepDev* __restrict__ steps, int nsteps,
-                                                         int total_blocks, T* __restrict__ arena, bool early) {
+                                                         int total_blocks, T* arena, bool early) {
   extern __shared__ int64_t tab[];
   __shared__ StepDev st;
   chain_trigger(early);
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(const StepDev* __restri
 
 template <typename T>
 __global__ void __launch_bounds__(kBodyThreads) k_splitk(const StepDev* __restrict__ steps, int nsteps,
-                                                         const T* __restrict__ arena, double2* __restrict__ partial) {
+                                                         const T* arena, double2* partial) {
   extern __shared__ int64_t tab[];
   __shared__ double red_re[kBodyThreads], red_im[kBodyThreads];
   splitk_body<T, SyncBlock>(steps, nsteps, arena, partial, blockIdx.x, tab, red_re, red_im);
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(kBodyThreads) k_splitk(const StepDev* __restri
 // sized for 4 blocks per SM (3 for the staged FP32 form, whose stages take more shared memory)
 template <typename T, bool kF32>
 __global__ void __launch_bounds__(kBodyThreads, 4) k_dot(const StepDev* __restrict__ steps, int nsteps,
-                                                      const T* __restrict__ arena, double2* __restrict__ partial) {
+                                                      const T* arena, double2* partial) {
   extern __shared__ int64_t tab[];
   __shared__ double red_re[kBodyThreads], red_im[kBodyThreads];
   dot_body<T, kF32, SyncBlock, kF32>(steps, nsteps, arena, partial, blockIdx.x, tab, red_re, red_im);
@@ -63,8 +63,8 @@ __global__ void __launch_bounds__(kBodyThreads, 4) k_dot(const StepDev* __restri
 
 template <typename T>
 __global__ void __launch_bounds__(kBodyThreads) k_splitk_done(const StepDev* __restrict__ steps, int nsteps,
-                                                              const double2* __restrict__ partial,
-                                                              T* __restrict__ arena, double2* __restrict__ scalars) {
+                                                              const double2* partial,
+                                                              T* arena, double2* scalars) {
   (void)nsteps;
   chain_wait();
   __shared__ double red_re[kBodyThreads], red_im[kBodyThreads];
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kBodyThreads) k_splitk_done(const StepDev* __r
 // the FP64 operand mode, FP32 otherwise).
 template <typename S>
 __global__ void __launch_bounds__(kBodyThreads, 4) k_perm(const PermDev* __restrict__ perms,
-                                                       const double* __restrict__ arena, char* __restrict__ base,
+                                                       const double* arena, char* base,
                                                        bool early) {
   extern __shared__ int64_t tab[];
   __shared__ PermSmem<S> sm;
@@ -90,17 +90,17 @@ __global__ void __launch_bounds__(kBodyThreads, 4) k_perm(const PermDev* __restr
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kBodyThreads) k_open(const FinalDev* __restrict__ fd, const T* __restrict__ arena,
-                                                       const double2* __restrict__ scalars,
-                                                       double* __restrict__ traces, double* __restrict__ partial) {
+__global__ void __launch_bounds__(kBodyThreads) k_open(const FinalDev* __restrict__ fd, const T* arena,
+                                                       const double2* scalars,
+                                                       double* traces, double* partial) {
   extern __shared__ int64_t tab[];
   __shared__ double red[kBodyThreads];
   chain_wait();
   open_body<T, SyncBlock>(fd, arena, scalars, traces, partial, blockIdx.x, gridDim.x, tab, red);
 }
 
-__global__ void k_final(const FinalDev* __restrict__ fd, const double2* __restrict__ scalars,
-                        const double* __restrict__ partial, double* __restrict__ result) {
+__global__ void k_final(const FinalDev* __restrict__ fd, const double2* scalars,
+                        const double* partial, double* result) {
   chain_wait();
   if (threadIdx.x == 0) final_body(fd, scalars, partial, result);
 }
@@ -108,10 +108,10 @@ __global__ void k_final(const FinalDev* __restrict__ fd, const double2* __restri
 // Both in one launch when one block covers the open tensor (always for Alg. II, whose result is the
 // product of scalars): one kernel less at the end of every evaluation's chain.
 template <typename T>
-__global__ void __launch_bounds__(kBodyThreads) k_open_final(const FinalDev* __restrict__ fd, const T* __restrict__ arena,
-                                                             const double2* __restrict__ scalars,
-                                                             double* __restrict__ traces, double* __restrict__ partial,
-                                                             double* __restrict__ result) {
+__global__ void __launch_bounds__(kBodyThreads) k_open_final(const FinalDev* __restrict__ fd, const T* arena,
+                                                             const double2* scalars,
+                                                             double* traces, double* partial,
+                                                             double* result) {
   extern __shared__ int64_t tab[];
   __shared__ double red[kBodyThreads];
   chain_wait();

@@ -11,7 +11,11 @@ cudaError_t set_kernel_smem_limits();
 // Launches of a program's chain of dependent kernels. Every kernel of the chain is launched with
 // programmatic stream serialization and waits (griddepcontrol.wait) before its first access to what
 // other kernels read or write, so its launch latency, descriptor loads and offset tables overlap the
-// end of the kernel before it. `early`: the kernel lets its successor start at once; set for short
+// end of the kernel before it. Such a kernel is resident while others still write the tensors that it is
+// going to read, and while others read what lay at their addresses before. So no pointer to data that another
+// kernel writes is __restrict__ here: that would promise memory that does not change while the kernel lives,
+// and allow non-coherent loads and loads moved above the wait. (Descriptors, uploaded before the chain
+// starts, may be.) `early`: the kernel lets its successor start at once; set for short
 // kernels only (chain_early), because a successor that waits for long holds shared memory and warps that
 // other streams could use.
 template <typename... KArgs, typename... Args>

@@ -241,8 +241,8 @@ int tc_gemm_splits(int64_t M, int64_t N, int64_t K, int kind) {
 namespace {
 
 // C[i] = sum over splits s (in order) of W[s][i] (compensated FP32 sum)
-__global__ void __launch_bounds__(kBodyThreads) k_split_sum(const float* __restrict__ W, int ksplit, int64_t n,
-                                                            float* __restrict__ C) {
+__global__ void __launch_bounds__(kBodyThreads) k_split_sum(const float* W, int ksplit, int64_t n,
+                                                            float* C) {
   chain_wait();
   split_sum_body(W, ksplit, n, C, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x));
 }

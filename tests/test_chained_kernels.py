@@ -1,0 +1,79 @@
+"""Kernels that are resident while their predecessors still run (launch_chained): what their source has
+to say for their reads to be ordered, and evaluations repeated until a disorder would show."""
+import os
+import re
+
+import numpy as np
+import pytest
+
+from paper_2103_11595_gb300 import ajf, workloads as W
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2103_11595_gb300", "csrc")
+DESCRIPTORS = {"StepDev", "PermDev", "FinalDev"}  # uploaded before a chain starts, written by no kernel
+
+
+def source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def restrict_params(text, function):
+    """Pointee types of the __restrict__ parameters of `function` where it is defined."""
+    found = [re.search(r"\b%s\(([^)]*)\)\s*\{" % function, text)]
+    assert found[0], function
+    return [t for t in re.findall(r"(\w+)\s*\*\s*__restrict__", found[0].group(1))]
+
+
+@pytest.mark.parametrize("name", ["kernels.cu", "dg_gemm.cu", "tc_gemm.cu"])
+def test_chained_kernels_promise_nothing_about_others_data(name):
+    """A __restrict__ pointer to data that a predecessor writes allows non-coherent loads, and loads
+    above the wait."""
+    text = source(name)
+    kernels = {k for call in re.findall(r"launch_chained\(([^;]*);", text) for k in re.findall(r"\bk_\w+", call)}
+    assert kernels
+    for k in sorted(kernels):
+        assert set(restrict_params(text, k)) <= DESCRIPTORS, k
+
+
+def test_shared_bodies_promise_nothing_about_others_data():
+    for name in ("bodies.cuh", "dg_gemm.cu"):
+        text = source(name)
+        for body in sorted(set(re.findall(r"\b(\w+_body|perm_tiles_\w+)\(const \w+[&*]", text))):
+            assert set(restrict_params(text, body)) <= DESCRIPTORS, body
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", ["f64", "f32", "bf16x6", "tf32x3", "bf16x3"])
+def test_repeated_evaluations_are_bitwise_equal(precision):
+    """The same plan and inputs, enqueued one by one and from a graph, always give the same bits (every
+    kernel sums in a fixed order), also with several circuits' chains side by side."""
+    insts = [W.mid(s) for s in (0, 3, 7)]
+    ctxs = [ajf.Context(0) for _ in insts]
+    try:
+        for graph in (False, True):
+            for c, inst in zip(ctxs, insts):
+                ajf.load_instance(c.handle, inst)
+                ajf.ajf_plan(c.handle, 2, precision=precision, trials=8, use_graph=graph)
+            first = [ajf.ajf_fidelity_alg2(c.handle)["S"] for c in ctxs]
+            for _ in range(40):
+                assert [ajf.ajf_fidelity_alg2(c.handle)["S"] for c in ctxs] == first
+            for _ in range(40):
+                assert [r["S"] for r in ajf.ajf_fidelity_batch([c.handle for c in ctxs], 2)] == first
+    finally:
+        for c in ctxs:
+            c.close()
+
+
+@pytest.mark.gpu
+def test_repeated_traces_are_bitwise_equal():
+    """A chain of short launches (small steps, split-K sums), each of which lets the next one start."""
+    inst = W.batching_circuit(1)
+    with ajf.Context(0) as c:
+        ajf.load_instance(c.handle, inst)
+        ajf.ajf_plan(c.handle, 1, trials=8)
+        n = inst.n_combinations()
+        ajf.ajf_fidelity_alg1(c.handle)
+        first = ajf.ajf_alg1_traces(c.handle, n)
+        for _ in range(100):
+            ajf.ajf_fidelity_alg1(c.handle)
+            assert np.array_equal(ajf.ajf_alg1_traces(c.handle, n), first)
