@@ -42,6 +42,29 @@ def test_shared_bodies_promise_nothing_about_others_data():
             assert set(restrict_params(text, body)) <= DESCRIPTORS, body
 
 
+def test_epilogue_lanes_wait_for_what_they_read():
+    """No lane of the GEMM's epilogue reads scales or accumulators on another lane's word (a shuffle
+    orders no memory)."""
+    epilogue = source("tc_gemm_dev.cuh").split("} else if (warp >= kEpiWarp0) {")[1].split("if (mine) {")[0]
+    assert epilogue.count("mbar_wait(") == 2
+    assert "if (lane == 0) w" not in epilogue and "__shfl_sync" not in epilogue
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("seed", range(10))
+def test_repeated_scaled_fp16_evaluations_are_bitwise_equal(seed):
+    """The mode whose epilogue also reads per-block scales that the GEMM copies in; the chain without and
+    with a graph, and a new context's first evaluation among the repeated ones."""
+    inst = W.mid(seed)
+    seen = set()
+    for k in range(4):
+        with ajf.Context(0) as c:
+            ajf.load_instance(c.handle, inst)
+            ajf.ajf_plan(c.handle, 2, precision="f16x3", trials=8, use_graph=k % 2 == 1)
+            seen |= {ajf.ajf_fidelity_alg2(c.handle)["S"] for _ in range(25)}
+    assert len(seen) == 1
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("precision", ["f64", "f32", "bf16x6", "tf32x3", "bf16x3"])
 def test_repeated_evaluations_are_bitwise_equal(precision):
