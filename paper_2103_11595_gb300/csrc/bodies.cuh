@@ -266,6 +266,9 @@ __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, in
   Sync::sync();
   const int64_t nout = int64_t(1) << st.rc, nk = int64_t(1) << st.rk;
   const bool one_chunk = c_ka == 1;  // (no chunk, rk = 0: lookup gives 0)
+  // the lanes of a warp that have an output: nout is a power of two and a warp's outputs are consecutive,
+  // so all of them, or the first nout of the one warp that has any
+  const unsigned act = nout < 32 ? (1u << nout) - 1u : 0xffffffffu;
   T* C = arena + st.c;
   with_operands(arena, st.a, st.fa, st.b, st.fb, [&](const auto* A, const auto* B) {
     using TA = typename std::remove_cv<typename std::remove_pointer<decltype(A)>::type>::type;
@@ -305,7 +308,6 @@ __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, in
         for (int j = 0; j < 4; ++j) {
           if (kk + j >= nk) break;
           // (votes: a branch that the whole warp takes together needs no reconvergence)
-          const unsigned act = __activemask();
           if (__any_sync(act, !is_zero(yr[j]))) {
             re = fma(widen(xr[j]), widen(yr[j]), re);
             im = fma(widen(xi[j]), widen(yr[j]), im);

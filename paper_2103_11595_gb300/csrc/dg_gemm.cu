@@ -235,6 +235,7 @@ __device__ __forceinline__ void digits_body(const PermDev& p, const S* src, char
   const int lanes = 1 << (p.tk - 3);               // units of one row of the tile
   chain_wait();
   __syncthreads();
+  const unsigned units = __ballot_sync(0xffffffffu, unit);  // lanes that take part in a row's reduction
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t r0 = (tile >> kt_bits) << p.tr, k0 = (tile & ((int64_t(1) << kt_bits) - 1)) << p.tk;
     if (tm.active) {
@@ -257,8 +258,7 @@ __device__ __forceinline__ void digits_body(const PermDev& p, const S* src, char
           const int at = tile_place((u << 3) | j);
           E = max(E, max(exp_field(tre[at]), exp_field(tim[at])));
         }
-        const unsigned mask = __activemask();
-        for (int o = 1; o < lanes; o <<= 1) E = max(E, __shfl_xor_sync(mask, E, o));
+        for (int o = 1; o < lanes; o <<= 1) E = max(E, __shfl_xor_sync(units, E, o));
       } else {
         for (int s = 0; s < p.strips; ++s) E = max(E, part[s * R + r]);
       }

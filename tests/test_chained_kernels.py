@@ -50,6 +50,13 @@ def test_epilogue_lanes_wait_for_what_they_read():
     assert "if (lane == 0) w" not in epilogue and "__shfl_sync" not in epilogue
 
 
+def test_warp_operations_name_their_lanes():
+    """A shuffle or vote over whichever lanes happen to be together drops the others' values: the masks
+    come from the conditions that the lanes are under."""
+    for name in os.listdir(CSRC):
+        assert "__activemask" not in source(name), name
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("seed", range(10))
 def test_repeated_scaled_fp16_evaluations_are_bitwise_equal(seed):
