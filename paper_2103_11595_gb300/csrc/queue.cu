@@ -236,7 +236,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_queue(const QPhase* __restrict_
       }
     }
   }
-  if (*sh.abort_flag) tc_drain_after_abort(kQSlots, kQBufs, wait_ns, status, sh, ring);
+  if (__any_sync(0xffffffffu, *sh.abort_flag != 0))
+    tc_drain_after_abort(kQSlots, kQBufs, wait_ns, status, sh, ring);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncwarp();
   __syncthreads();

@@ -92,7 +92,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
   TcRing ring;
   const uint32_t nwork = static_cast<uint32_t>(p.tiles) * static_cast<uint32_t>(p.ksplit);
   tc_gemm_terms<BN, kKind, kT>(p, blockIdx.x, nwork, gridDim.x, sh, ring);
-  if (*sh.abort_flag) tc_drain_after_abort(p.slots, p.bufs, p.wait_ns, p.status, sh, ring);
+  if (__any_sync(0xffffffffu, *sh.abort_flag != 0))
+    tc_drain_after_abort(p.slots, p.bufs, p.wait_ns, p.status, sh, ring);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   // __syncthreads (bar.sync, the aligned form) must be executed by all threads of a warp
   // together; warps 0 and 1 get here diverged (lane 0 ran the producer / MMA loop, lanes 1-31 came

@@ -560,7 +560,8 @@ __device__ __forceinline__ bool tc_gemm_items(const TcParams& p, uint32_t wi0, u
 
 // After an abort (the abort flag set), before the block releases its shared memory and TMEM: the
 // producer waits (bounded) until the loads it issued have landed -- the last min(issued, S) slots;
-// earlier ones were consumed -- and the MMA issuer until every MMA it issued has completed.
+// earlier ones were consumed -- and the MMA issuer until every MMA it issued has completed. The lanes
+// of a warp call it together.
 __device__ __forceinline__ void tc_drain_after_abort(int slots, int nbufs, unsigned long long wait_ns, int* status,
                                                      const TcShared& sh, const TcRing& r) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -568,7 +569,7 @@ __device__ __forceinline__ void tc_drain_after_abort(int slots, int nbufs, unsig
   if (warp == 0 && lane == 0 && r.issued > 0) {
     const uint32_t first = r.issued > S ? r.issued - S : 0u;
     for (uint32_t i = first; i < r.issued; ++i) mbar_wait(sh.full0 + 8 * (i % S), (i / S) & 1u, wait_ns, status, 15);
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {  // a commit tracks what its own thread issued: the issuer's lane
     if (r.any) {
       mma_commit(sh.drain0);
       mbar_wait(sh.drain0, 0u, wait_ns, status, 16);

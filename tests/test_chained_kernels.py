@@ -57,6 +57,16 @@ def test_warp_operations_name_their_lanes():
         assert "__activemask" not in source(name), name
 
 
+def test_drain_commits_from_the_lane_that_issued():
+    """A commit tracks the MMAs of the thread that executes it: wherever an elected lane issues them, an
+    elected lane commits them, also in the drain after an abort."""
+    drain = source("tc_gemm_dev.cuh").split("void tc_drain_after_abort(")[1]
+    issuer = drain[:drain.index("mma_commit(")].rsplit("else if", 1)[1]
+    assert "warp == 1 && elect_one()" in issuer and "lane" not in issuer
+    for name in ("tc_gemm.cu", "queue.cu"):  # and every lane of the warp is there to elect it
+        assert re.search(r"if \(__any_sync\(0xffffffffu, \*sh\.abort_flag != 0\)\)\s*tc_drain_after_abort", source(name))
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("seed", range(10))
 def test_repeated_scaled_fp16_evaluations_are_bitwise_equal(seed):
