@@ -62,11 +62,13 @@ using namespace dg;
 constexpr int kTileElems = 2048;  // complex elements of a gather tile (at most)
 constexpr int kDigThreads = 512;  // gather threads: 256 units of 8 elements per plane
 
-// The exponent field (FP64 encoding) of a source value; zero and subnormal values give 0.
+// The exponent field (FP64 encoding) of a source value; zero and subnormal values give 0, infinities and
+// NaN kNonFinite.
+constexpr int kNonFinite = 0x7FF;
 __device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 __device__ __forceinline__ int exp_field(float x) {
   const int f = (__float_as_uint(x) >> 23) & 0xFF;
-  return f ? f + (1023 - 127) : 0;
+  return f == 0xFF ? kNonFinite : (f ? f + (1023 - 127) : 0);
 }
 __device__ __forceinline__ uint64_t f64_bits(double x) { return static_cast<uint64_t>(__double_as_longlong(x)); }
 // exact, without the FP64 pipe
@@ -371,9 +373,15 @@ __device__ __forceinline__ void dg_layout(uint8_t* slots, uint8_t* bars, DgShare
 }
 static_assert(16 * kDgMaxSlots + 16 * kDgMaxBufs + 16 <= kDgControl, "control region");
 
+// Exponent of a sum's unit that stands for NaN: a row with an infinity or a NaN has no digits, so all of
+// its products are NaN. (Added once per side, on exponents below 2^12.)
+constexpr int kNanUnit = 1 << 16;
+__device__ __forceinline__ int unit_field(int f) { return f == kNonFinite ? kNanUnit : f; }
+
 // acc 2^(e) rounded to nearest (even) in FP64, e = exponent of acc's unit: integer arithmetic only
 // (a 64-bit conversion instruction runs at the FP64 pipe's rate). Below the normal range: 0.
 __device__ __forceinline__ double fixed_to_f64(int64_t acc, int e) {
+  if (e > kNanUnit / 2) return __longlong_as_double(0x7FF8000000000000ll);
   const uint64_t s = static_cast<uint64_t>(acc) & 0x8000000000000000ull;
   uint64_t u = acc < 0 ? static_cast<uint64_t>(-acc) : static_cast<uint64_t>(acc);
   if (u == 0) return 0.0;
@@ -387,6 +395,7 @@ __device__ __forceinline__ double fixed_to_f64(int64_t acc, int e) {
   return __longlong_as_double(static_cast<long long>(s | ((static_cast<uint64_t>(f - 1) << 52) + m)));
 }
 __device__ __forceinline__ float fixed_to_f32(int64_t acc, int e) {
+  if (e > kNanUnit / 2) return __uint_as_float(0x7FC00000u);
   const uint32_t s = acc < 0 ? 0x80000000u : 0u;
   uint64_t u = acc < 0 ? static_cast<uint64_t>(-acc) : static_cast<uint64_t>(acc);
   if (u == 0) return 0.0f;
@@ -564,7 +573,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
       const int64_t n = static_cast<int64_t>(ty) * kTileRows + 32 * q + lane;
       const int m0 = tx * BC + h * COLS;
       if (n < p.N) {
-        const int e0 = p.ey[n] - 2 * (1023 + 7) - p.sh0;
+        const int e0 = unit_field(p.ey[n]) - 2 * (1023 + 7) - p.sh0;
         const bool part = p.ksplit > 1;
         const int64_t at = (part ? static_cast<int64_t>(wi / tiles) * p.M * p.N : 0) + m0 * p.N + n;
         double* wd = part ? p.ws + at : static_cast<double*>(p.C) + at;  // FP64 partials, or an FP64 result
@@ -575,7 +584,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
           int e;
           // (volatile: hoisted above the loop, the loads would not leave enough registers)
           asm volatile("ld.global.s32 %0, [%1];" : "=r"(e) : "l"(exm + j));
-          e += e0;
+          e = unit_field(e) + e0;
           if (sizeof(Out) == 8 || part) {
             *wd = fixed_to_f64(acc[j], e);
             wd += p.N;

@@ -63,7 +63,9 @@ struct Piece {
 
 // X + bias for an FP64 value given by its bits and its row's largest exponent field E (>= its own):
 // digit t >= 1 is then ((Y >> (54 - 9 t)) & 511) - 256 and d_0 = Y >> 54. A zero exponent field (zero
-// and subnormal values, below 2^-1022) counts as zero. terms = 6 (the bias of the digits 1..5).
+// and subnormal values, below 2^-1022) counts as zero. terms = 6 (the bias of the digits 1..5). An
+// infinity or a NaN gives digits without a meaning: its row's exponent says so, and the product's epilogue
+// writes NaN for the row.
 __host__ __device__ inline int64_t biased_fixed(uint64_t bits, int row_field, int terms) {
   const int f = static_cast<int>((bits >> 52) & 0x7FF);
   int64_t x = 0;

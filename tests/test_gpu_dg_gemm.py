@@ -62,6 +62,28 @@ def test_digit_gemm_against_extended_precision(precision, shape):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(16, 16, 8), (16, 32, 16), (32, 128, 64), (64, 64, 512), (16, 32, 4096)])
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_non_finite_rows_stay_non_finite(precision, shape):
+    """A row with an infinity or a NaN anywhere gives NaN products, and no other row is touched."""
+    M, N, K = shape
+    A, B = operands(M, N, K, "normal", 3)
+    clean = ajf.ajf_selftest_digit_gemm(0, precision, A, B)
+    A, B = A.copy(), B.copy()
+    A.real[1, K - 1] = np.inf
+    A.imag[M - 1, 0] = np.nan
+    B.imag[2, K // 2] = -np.inf
+    B.real[N - 1, 1] = np.nan
+    bad = np.zeros((M, N), bool)
+    bad[[1, M - 1]] = True
+    bad[:, [2, N - 1]] = True
+    for order in (0, 1, 2):
+        C = ajf.ajf_selftest_digit_gemm(0, precision, A, B, order=order)
+        assert np.isnan(C.real[bad]).all() and np.isnan(C.imag[bad]).all()
+        assert np.array_equal(C[~bad], clean[~bad])
+
+
+@pytest.mark.gpu
 def test_fixed_arena_takes_plans_that_only_digits_outgrow():
     """A plan over the 64 MiB of the no-allocation call because of its digit operands runs there with
     CUDA-core GEMMs, and the context's own program is unchanged."""
