@@ -223,6 +223,8 @@ __device__ __forceinline__ bool is_zero(double x) {
   return ((__double2hiint(x) << 1) | __double2loint(x)) == 0;
 }
 __device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
+__device__ __forceinline__ bool is_finite(double x) { return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000; }
+__device__ __forceinline__ bool is_finite(float x) { return (__float_as_uint(x) & 0x7F800000u) != 0x7F800000u; }
 // FP32 to FP64, exact, on the integer pipe (the conversion instruction takes the FP64 pipe as long as a
 // multiply-add does); subnormal and non-finite values through the instruction.
 __device__ __forceinline__ double widen(double x) { return x; }
@@ -307,12 +309,14 @@ __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, in
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           if (kk + j >= nk) break;
-          // (votes: a branch that the whole warp takes together needs no reconvergence)
-          if (__any_sync(act, !is_zero(yr[j]))) {
+          // (votes: a branch that the whole warp takes together needs no reconvergence). A zero is
+          // skipped only beside finite factors: 0 times an infinity or a NaN is NaN
+          const bool keep = !is_finite(xr[j]) || !is_finite(xi[j]);
+          if (__any_sync(act, keep || !is_zero(yr[j]))) {
             re = fma(widen(xr[j]), widen(yr[j]), re);
             im = fma(widen(xi[j]), widen(yr[j]), im);
           }
-          if (__any_sync(act, !is_zero(yi[j]))) {
+          if (__any_sync(act, keep || !is_zero(yi[j]))) {
             re = fma(-widen(xi[j]), widen(yi[j]), re);
             im = fma(widen(xr[j]), widen(yi[j]), im);
           }
