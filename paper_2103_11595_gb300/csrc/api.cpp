@@ -112,6 +112,7 @@ struct ajf_ctx {
   std::vector<char> alt_image;
   int64_t alt_gen = -1;  // prog_gen it was made for
   double plain_budget = 0;  // > 0: the program has CUDA-core GEMMs to meet this memory budget
+  bool prog_smallest = false;  // no other GEMMs or path make the program smaller (and it was over its budget)
   // tensor-core GEMM launches prepared on the host for (program, arena); index = launch index.
   // One set for the context's own arena, one for the fixed arena of ajf_fidelity_noalloc, so
   // that alternating the two paths re-encodes nothing.
@@ -1170,12 +1171,14 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
   pkey.push_back(c->tc_device ? 1 : 0);
   pkey.push_back(o.slice_bonds);
   if (o.slice_bonds == AJF_SLICE_AUTO) pkey.push_back(static_cast<int64_t>(budget));
-  // (a cached program with CUDA-core GEMMs in place of digit ones stands for budgets up to the one
-  // that asked for it, and one over this budget is lowered anew if that may make it fit)
+  // A cached program with CUDA-core GEMMs in place of digit ones stands for the budgets between its
+  // arena and the one that asked for it; one over this budget is lowered anew, unless every way to make
+  // it smaller was tried. (Under AJF_SLICE_AUTO the budget is part of the key.)
   const bool may_shrink = o.precision <= AJF_PREC_F32 && c->tc_device && o.lowering != AJF_LOWER_PERSISTENT;
-  const bool prog_hit = c->prog_valid && pkey == c->prog_key &&
-                        (c->plain_budget > 0 ? budget <= c->plain_budget
-                                             : !may_shrink || static_cast<double>(c->prog.arena_bytes) <= budget);
+  const bool stands = !may_shrink || o.slice_bonds == AJF_SLICE_AUTO ||
+                      (static_cast<double>(c->prog.arena_bytes) > budget ? c->prog_smallest
+                                                                        : c->plain_budget <= 0 || budget <= c->plain_budget);
+  const bool prog_hit = c->prog_valid && pkey == c->prog_key && stands;
   bool cached = prog_hit;
   if (!prog_hit) {
     drop_graph(c);
@@ -1244,20 +1247,45 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
         }
       };
       if (score_err == cudaSuccess) lower_path(true);
-      // The digit operands of the F64 and F32 modes take up to 1.5 times the memory of the CUDA-core
+      // The digit operands of the F64 and F32 modes take 1.5 to 2 times the memory of the CUDA-core
       // GEMMs', and the planner's model prefers wider paths with them. A plan over the budget is
-      // tried again with CUDA-core GEMMs, on the same path and then on one planned for them.
+      // tried again with CUDA-core GEMMs, on the same path and then on one planned for them; the first
+      // that fits is taken, or else the smallest.
       auto over = [&] { return !lowered || static_cast<double>(c->prog.arena_bytes) > budget; };
       c->plain_budget = 0;
+      c->prog_smallest = false;
       if (score_err == cudaSuccess && may_shrink && over()) {
-        c->plain_budget = budget;
-        lower_path(false);
-        if (over()) {
-          c->path_valid = false;  // the path below belongs to this budget only
-          pp.tensor_cores = false;
-          c->path_full = plan_path(full, pp);
-          if (score_err == cudaSuccess) lower_path(false);
+        struct Lowered {
+          Path path_full, path;
+          Network net;
+          std::vector<int> labels;
+          Program prog;
+          bool lowered = false, plain = false, own = false;
+        };
+        Lowered best;
+        auto keep = [&](bool plain, bool own) {
+          best = Lowered{c->path_full, std::move(c->path), std::move(c->net), std::move(c->bond_labels), std::move(c->prog),
+                         lowered, plain, own};
+        };
+        keep(false, false);
+        for (int own = 0; own < 2 && score_err == cudaSuccess; ++own) {
+          if (own) {
+            pp.tensor_cores = false;
+            c->path_full = plan_path(full, pp);
+          }
+          lower_path(false);
+          if (!over() || (lowered && (!best.lowered || c->prog.arena_bytes < best.prog.arena_bytes))) keep(true, own != 0);
+          if (best.lowered && static_cast<double>(best.prog.arena_bytes) <= budget) break;
         }
+        c->path_full = std::move(best.path_full);
+        c->path = std::move(best.path);
+        c->net = std::move(best.net);
+        c->bond_labels = std::move(best.labels);
+        c->prog = std::move(best.prog);
+        lowered = best.lowered;
+        if (best.own) c->path_valid = false;  // this path belongs to this budget only
+        c->plain_budget = best.plain ? budget : 0;
+        c->prog_smallest = over();
       }
       c->bond_leaves.clear();
       for (size_t l = 0; l < full.leaf_labels.size(); ++l) {

@@ -112,3 +112,31 @@ def test_budget_between_the_two_gemms_keeps_the_plan(precision):
         assert tight["n_tc_gemms"] == 0 and tight["arena_bytes"] <= 0.96 * roomy["arena_bytes"]
         again = ajf.ajf_plan(c.handle, 2, precision=precision, trials=8)
         assert again["n_tc_gemms"] > 0 and again["arena_bytes"] == roomy["arena_bytes"]
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_plans_do_not_depend_on_the_budgets_before(precision):
+    """In one context, plans for falling and rising budgets are those of fresh contexts: as small, or
+    refused as over the budget with the smallest arena that any of the GEMMs and paths needs."""
+    inst = W.mid(0)
+
+    def plan(c, budget):
+        try:
+            i = ajf.ajf_plan(c.handle, 2, precision=precision, trials=8, mem_budget_bytes=budget)
+            return i["arena_bytes"], i["n_tc_gemms"]
+        except ajf.AjfError as e:
+            assert e.status == ajf.AJF_E_BUDGET
+            return "over budget", str(e).split("bytes")[0]
+
+    with ajf.Context(-1) as c:
+        ajf.load_instance(c.handle, inst)
+        roomy = plan(c, 1e18)[0]
+        for f in (0.96, 0.85, 0.8, 0.3, 0.8, 0.96, 0.2, 1.0):
+            with ajf.Context(-1) as fresh:
+                ajf.load_instance(fresh.handle, inst)
+                want = plan(fresh, f * roomy)
+            assert plan(c, f * roomy) == want, f
+        over = [plan(c, 1.0)[1], plan(c, 0.3 * roomy)[1]]
+        assert over[0] == over[1]  # the smallest, and kept: nothing is left to try
+        smallest = float(over[0].split("needs")[1])
+        assert plan(c, smallest)[0] == smallest and plan(c, smallest - 1)[0] == "over budget"
