@@ -1231,26 +1231,28 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
         }
       };
       bool lowered = false;
-      auto lower_path = [&](bool digits) {
+      const bool slice_auto = o.slice_bonds == AJF_SLICE_AUTO;
+      auto lower_path = [&](bool digits, bool slice) {  // slice: under AJF_SLICE_AUTO, as many labels as needed
         int count = o.slice_bonds > 0 ? o.slice_bonds : 0;
-        if (o.slice_bonds == AJF_SLICE_AUTO) count = std::max(0, c->path_full.width - (kMaxBits - 2));
+        if (slice_auto && slice) count = std::max(0, c->path_full.width - (kMaxBits - 2));
         for (;;) {
           apply_slices(std::min(count, static_cast<int>(AJF_MAX_SLICE_BONDS)));
           lowered = c->path.width <= kMaxBits - 2;
           if (lowered)
             c->prog = lower(c->net, c->path, o.precision, c->in.packed.size() / 2, c->tc_device,
                             o.lowering == AJF_LOWER_PERSISTENT, digits);
-          if (o.slice_bonds != AJF_SLICE_AUTO) break;
+          if (!slice_auto || !slice) break;
           if (lowered && static_cast<double>(c->prog.arena_bytes) <= budget) break;
           if (count >= AJF_MAX_SLICE_BONDS || static_cast<int>(c->bond_labels.size()) < count) break;
           ++count;
         }
       };
-      if (score_err == cudaSuccess) lower_path(true);
+      if (score_err == cudaSuccess) lower_path(true, !may_shrink);
       // The digit operands of the F64 and F32 modes take 1.5 to 2 times the memory of the CUDA-core
       // GEMMs', and the planner's model prefers wider paths with them. A plan over the budget is
       // tried again with CUDA-core GEMMs, on the same path and then on one planned for them; the first
-      // that fits is taken, or else the smallest.
+      // that fits is taken, or else the smallest. Under AJF_SLICE_AUTO the unsliced plans come first
+      // (what fits unsliced is not sliced: single-run calls take no sliced plan), then the sliced ones.
       auto over = [&] { return !lowered || static_cast<double>(c->prog.arena_bytes) > budget; };
       c->plain_budget = 0;
       c->prog_smallest = false;
@@ -1268,14 +1270,23 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
                          lowered, plain, own};
         };
         keep(false, false);
-        for (int own = 0; own < 2 && score_err == cudaSuccess; ++own) {
-          if (own) {
-            pp.tensor_cores = false;
-            c->path_full = plan_path(full, pp);
+        Path paths[2] = {c->path_full, {}};  // planned for digit products, and for CUDA-core GEMMs
+        bool planned_own = false;
+        for (int slice = 0; slice < (slice_auto ? 2 : 1); ++slice) {
+          for (int v = slice ? 0 : 1; v < 3; ++v) {  // digits, CUDA-core GEMMs, the same on their own path
+            const int own = v == 2;
+            pp.tensor_cores = !own;
+            if (own && !planned_own) {
+              paths[1] = plan_path(full, pp);
+              planned_own = true;
+            }
+            if (score_err != cudaSuccess) break;
+            c->path_full = paths[own];
+            lower_path(v == 0, slice != 0);
+            if (!over() || (lowered && (!best.lowered || c->prog.arena_bytes < best.prog.arena_bytes))) keep(v > 0, own != 0);
+            if (best.lowered && static_cast<double>(best.prog.arena_bytes) <= budget) break;
           }
-          lower_path(false);
-          if (!over() || (lowered && (!best.lowered || c->prog.arena_bytes < best.prog.arena_bytes))) keep(true, own != 0);
-          if (best.lowered && static_cast<double>(best.prog.arena_bytes) <= budget) break;
+          if (score_err != cudaSuccess || (best.lowered && static_cast<double>(best.prog.arena_bytes) <= budget)) break;
         }
         c->path_full = std::move(best.path_full);
         c->path = std::move(best.path);

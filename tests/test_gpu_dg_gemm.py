@@ -140,3 +140,28 @@ def test_plans_do_not_depend_on_the_budgets_before(precision):
         assert over[0] == over[1]  # the smallest, and kept: nothing is left to try
         smallest = float(over[0].split("needs")[1])
         assert plan(c, smallest)[0] == smallest and plan(c, smallest - 1)[0] == "over budget"
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_auto_slicing_leaves_plans_whole_that_fit_with_either_gemm(precision):
+    """AJF_SLICE_AUTO slices nothing while some unsliced plan fits the budget (a sliced plan is refused by
+    the single-run calls), and digit products' plans beyond that."""
+    inst = W.mid(0)
+
+    def plan(budget, **kw):
+        with ajf.Context(-1) as c:
+            ajf.load_instance(c.handle, inst)
+            info = ajf.ajf_plan(c.handle, 2, precision=precision, trials=8, mem_budget_bytes=budget, **kw)
+            ajf.ajf_check_plan(c.handle)
+        return info
+
+    roomy = plan(1e18)["arena_bytes"]
+    with pytest.raises(ajf.AjfError) as e:
+        plan(1.0)
+    smallest = float(str(e.value).split("needs")[1].split("bytes")[0])
+    assert smallest < roomy
+    for budget in (roomy, roomy - 1, smallest):
+        auto, plain = plan(budget, slice_bonds="auto"), plan(budget)
+        assert auto["n_sliced_bonds"] == 0 and auto["arena_bytes"] == plain["arena_bytes"] <= budget
+    tight = plan(smallest - 1, slice_bonds="auto")
+    assert tight["n_sliced_bonds"] == 1 and tight["n_tc_gemms"] > 0 and tight["arena_bytes"] < smallest
