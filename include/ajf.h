@@ -376,21 +376,35 @@ ajf_status ajf_fidelity_alg2(ajf_ctx *ctx, double eps, ajf_result *out);
  * It runs the same device program as ajf_fidelity_alg1 (alg = 1) / ajf_fidelity_alg2 (alg = 2),
  * with the same results, but in a fixed device arena of 64 MiB that libajf declares as a static
  * __device__ array: every GPU that loads the library holds those 64 MiB until the process exits.
+ * Plans of the F64 and F32 modes whose arena (ajf_workspace_size) exceeds 64 MiB run a program with
+ * CUDA-core GEMMs instead, which needs less memory: it computes the same F_J and traces, rounded
+ * differently, and slower. ajf_plan lowers it on the plan's own path; where it only fits on a path
+ * planned for it, ajf_prepare_noalloc plans that path.
  * It calls no cudaMalloc, cudaFree, cudaMallocHost or other allocating routine; inputs are copied
  * from the context's host memory and the result is read back synchronously. The context's own
  * arena, CUDA graph and Alg. I trace buffer are not touched (ajf_alg1_traces still returns the
  * last ajf_fidelity_alg1 result).
  * The arena's device address is looked up (cudaGetSymbolAddress, with the device current) by
  * ajf_create for every device context, which is also when the GPU reserves the array, so a
- * reservation failure surfaces there and this call itself performs no set-up. A context created
+ * reservation failure surfaces there and this call itself performs no set-up -- except on a plan
+ * that needs ajf_prepare_noalloc, when that call was left out. A context created
  * before a cudaDeviceReset keeps the old address: create a new context after a reset.
  * All calls on a device share the one arena and it keeps the last call's contents (the call
  * rewrites everything it reads, and zeroes its status words first). Calls whose device work
  * overlaps -- from different threads or different streams of one device -- race on the arena
  * and must be serialised by the caller.
  * Errors: AJF_E_ARG (alg, eps or out), AJF_E_STATE (no plan for `alg`, host-only context),
- * AJF_E_NOMEM (the plan's arena, ajf_workspace_size, exceeds 64 MiB), AJF_E_CUDA, AJF_E_TIMEOUT. */
+ * AJF_E_NOMEM (the plan's arena, ajf_workspace_size, exceeds 64 MiB, and so does every program that
+ * may stand in for it), AJF_E_CUDA, AJF_E_TIMEOUT. */
 ajf_status ajf_fidelity_noalloc(ajf_ctx *ctx, int alg, double eps, ajf_result *out);
+
+/* Host-side preparation of ajf_fidelity_noalloc for the current plan (no device work): after it that
+ * call only enqueues. It plans (as long as ajf_plan takes) for an F64 or F32 plan that fits the fixed
+ * arena only with CUDA-core GEMMs on a path of their own, and returns at once for every other plan.
+ * ajf_fidelity_noalloc prepares itself where this call was left out.
+ * Errors: AJF_E_ARG (NULL), AJF_E_STATE (no plan, host-only context, sliced plan), AJF_E_NOMEM (the
+ * plan does not fit the fixed arena: ajf_fidelity_noalloc would fail the same way). */
+ajf_status ajf_prepare_noalloc(ajf_ctx *ctx);
 
 /* After ajf_fidelity_alg1: copy the traces t_i = tr(U^dagger E_i) to `traces` (host, 2*count
  * doubles, interleaved), in enumeration order (lexicographic over noises in the order added,

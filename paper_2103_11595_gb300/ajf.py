@@ -131,6 +131,7 @@ def lib() -> ctypes.CDLL:
             "ajf_fidelity_batch": (I32, [ctypes.POINTER(P), ctypes.c_int, ctypes.c_int, D, ctypes.POINTER(Result)]),
             "ajf_version": (ctypes.c_char_p, []),
             "ajf_selftest_gemm": (I32, [ctypes.c_int, ctypes.c_int, ctypes.c_int, I64, I64, I64, P, P, P]),
+            "ajf_prepare_noalloc": (I32, [P]),
             "ajf_fidelity_noalloc": (I32, [P, ctypes.c_int, D, ctypes.POINTER(Result)]),
             "ajf_selftest_split_gemm": (I32, [ctypes.c_int, ctypes.c_int, I64, I64, I64, P, P, P]),
             "ajf_selftest_digit_gemm": (I32, [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, I64, I64, I64, P,
@@ -334,6 +335,12 @@ def ajf_fidelity_alg2(ctx, eps: float = -1.0) -> dict:
     r = Result()
     _check(ctx, lib().ajf_fidelity_alg2(ctx, float(eps), ctypes.byref(r)))
     return r.as_dict()
+
+
+def ajf_prepare_noalloc(ctx) -> None:
+    """Host-side preparation of ajf_fidelity_noalloc for the current plan; raises AJF_E_NOMEM when the
+    plan does not fit the fixed arena."""
+    _check(ctx, lib().ajf_prepare_noalloc(ctx))
 
 
 def ajf_fidelity_noalloc(ctx, alg: int, eps: float = -1.0) -> dict:

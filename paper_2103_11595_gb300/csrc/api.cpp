@@ -108,9 +108,10 @@ struct ajf_ctx {
   std::vector<int64_t> prog_key;
   bool prog_valid = false;
   int64_t prog_gen = 0;  // bumped whenever a new program is lowered
-  ajf::Program alt_prog;  // fixed-arena program of an F64 / F32 plan that outgrows that arena (plan_fixed_arena)
+  ajf::Program alt_prog;  // fixed-arena program of an F64 / F32 plan that outgrows that arena (prepare_fixed_arena)
   std::vector<char> alt_image;
-  int64_t alt_gen = -1;  // prog_gen it was made for
+  int64_t alt_gen = -1;       // prog_gen it was made for
+  bool alt_searched = false;  // a path was also planned for it
   double plain_budget = 0;  // > 0: the program has CUDA-core GEMMs to meet this memory budget
   bool prog_smallest = false;  // no other GEMMs or path make the program smaller (and it was over its budget)
   // tensor-core GEMM launches prepared on the host for (program, arena); index = launch index.
@@ -1058,25 +1059,50 @@ PlanParams plan_params(const ajf_plan_opts& o, bool tensor_cores) {
   return pp;
 }
 
-// The program of the fixed arena (ajf_fidelity_noalloc): the context's own when it fits, else, for
-// the F64 and F32 modes (whose digit operands take more memory), one with CUDA-core GEMMs -- on the
-// same path, or on one planned for them. Kept until the next plan; `alt.prog.arena_bytes` is the
-// smallest found.
-void plan_fixed_arena(ajf_ctx* c) {
-  if (c->alt_gen == c->prog_gen) return;
-  auto consider = [&](const Path& path) {
-    Program p = lower(c->net, path, c->opts.precision, c->in.packed.size() / 2, c->tc_device, false, false);
-    if (c->alt_gen != c->prog_gen || p.arena_bytes < c->alt_prog.arena_bytes) c->alt_prog = std::move(p);
-    c->alt_gen = c->prog_gen;
+// Key of the paths planned for CUDA-core GEMMs in the process-wide cache.
+std::vector<int64_t> cuda_core_key(std::vector<int64_t> key) {
+  key[0] += 2;  // (the algorithm, 1 or 2, of every other key)
+  return key;
+}
+
+// Whether ajf_fidelity_noalloc runs another program than the context's: plans of the F64 and F32 modes
+// over the fixed arena, whose digit operands take more memory than CUDA-core GEMMs.
+bool outgrows_fixed_arena(const ajf_ctx* c) {
+  return c->device >= 0 && c->tc_device && c->opts.precision <= AJF_PREC_F32 &&
+         c->opts.lowering != AJF_LOWER_PERSISTENT && !multi_run(c) && c->prog.arena_bytes > kStaticArenaBytes;
+}
+
+// That program: CUDA-core GEMMs on the plan's own path (made by ajf_plan: under 2 ms) or, with `search`, on
+// one planned for them if that one alone fits (as long as planning takes). Kept until the next plan;
+// alt_prog.arena_bytes is the smallest found.
+void prepare_fixed_arena(ajf_ctx* c, bool search) {
+  auto lower_plain = [&](const Path& path) {
+    return lower(c->net, path, c->opts.precision, c->in.packed.size() / 2, c->tc_device, false, false);
   };
-  consider(c->path);
-  if (c->alt_prog.arena_bytes > kStaticArenaBytes) {
-    PlanParams pp = plan_params(c->opts, false);
-    if (pp.planner == AJF_PLANNER_LEARNED) pp.planner = AJF_PLANNER_AUTO;
-    const Path path = plan_path(c->net, pp);
-    if (path.width <= kMaxBits - 2) consider(path);
+  if (c->alt_gen != c->prog_gen) {
+    c->alt_gen = -1;
+    c->alt_prog = lower_plain(c->path);
+    c->alt_image = descriptor_image(c->alt_prog);
+    c->alt_searched = false;
+    c->alt_gen = c->prog_gen;
   }
-  c->alt_image = descriptor_image(c->alt_prog);
+  if (!search || c->alt_searched || c->alt_prog.arena_bytes <= kStaticArenaBytes) return;
+  PlanParams pp = plan_params(c->opts, false);
+  std::vector<int64_t> key = cuda_core_key(c->plan_key);
+  if (pp.planner == AJF_PLANNER_LEARNED) pp.planner = AJF_PLANNER_AUTO;
+  Path path;
+  if (!shared_path_lookup(key, &path)) {
+    path = plan_path(c->net, pp);
+    shared_path_store(key, path);
+  }
+  if (path.width <= kMaxBits - 2) {
+    Program p = lower_plain(path);
+    if (p.arena_bytes < c->alt_prog.arena_bytes) {
+      c->alt_image = descriptor_image(p);
+      c->alt_prog = std::move(p);
+    }
+  }
+  c->alt_searched = true;
 }
 
 ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_info* info) {
@@ -1277,7 +1303,11 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
             const int own = v == 2;
             pp.tensor_cores = !own;
             if (own && !planned_own) {
-              paths[1] = plan_path(full, pp);
+              const bool shared = o.planner != AJF_PLANNER_LEARNED;
+              if (!shared || !shared_path_lookup(cuda_core_key(key), &paths[1])) {
+                paths[1] = plan_path(full, pp);
+                if (shared) shared_path_store(cuda_core_key(key), paths[1]);
+              }
               planned_own = true;
             }
             if (score_err != cudaSuccess) break;
@@ -1382,6 +1412,12 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
   for (int j : slice_noises) c->slice_leaves.push_back(c->net.noise_leaf[j]);
   c->planned = true;
   c->plan_gen++;
+  if (outgrows_fixed_arena(c)) {
+    try {
+      prepare_fixed_arena(c, false);
+    } catch (const std::exception&) {  // ajf_prepare_noalloc tries again, and reports
+    }
+  }
   c->err.clear();
   return AJF_OK;
 }
@@ -1707,6 +1743,30 @@ ajf_status ajf_fidelity(ajf_ctx* c, double eps, ajf_result* out) {
   return fidelity(c, c->alg, eps, out);
 }
 
+namespace {
+ajf_status fixed_arena_full(ajf_ctx* c, size_t bytes) {
+  return fail(c, AJF_E_NOMEM, "plan needs " + std::to_string(bytes) + " bytes of device memory; the fixed " +
+                                  "arena of ajf_fidelity_noalloc holds " + std::to_string(kStaticArenaBytes) + " bytes");
+}
+}  // namespace
+
+ajf_status ajf_prepare_noalloc(ajf_ctx* c) {
+  if (!c) return AJF_E_ARG;
+  if (!c->planned) return fail(c, AJF_E_STATE, "no plan");
+  if (c->device < 0) return fail(c, AJF_E_STATE, "host-only context (device -1) cannot run the contraction");
+  if (multi_run(c)) return fail(c, AJF_E_STATE, "a sliced plan runs through ajf_fidelity_alg1/2 / ajf_fidelity only");
+  size_t bytes = c->prog.arena_bytes;
+  if (outgrows_fixed_arena(c)) {
+    try {
+      prepare_fixed_arena(c, true);
+    } catch (const std::exception& ex) {
+      return fail(c, AJF_E_NOMEM, std::string("planning for the fixed arena failed: ") + ex.what());
+    }
+    bytes = c->alt_prog.arena_bytes;
+  }
+  return bytes > kStaticArenaBytes ? fixed_arena_full(c, bytes) : AJF_OK;
+}
+
 ajf_status ajf_fidelity_noalloc(ajf_ctx* c, int alg, double eps, ajf_result* out) {
   if (!c) return AJF_E_ARG;
   if (!out) return fail(c, AJF_E_ARG, "out is NULL");
@@ -1727,21 +1787,14 @@ ajf_status ajf_fidelity_noalloc(ajf_ctx* c, int alg, double eps, ajf_result* out
       if (c) swap();
     }
   } alt;
-  if (c->prog.arena_bytes > kStaticArenaBytes && c->opts.precision <= AJF_PREC_F32 && c->prog.tensor_cores > 0) {
-    try {
-      plan_fixed_arena(c);
-    } catch (const std::exception& ex) {
-      return fail(c, AJF_E_NOMEM, std::string("planning for the fixed arena failed: ") + ex.what());
-    }
-    if (c->alt_prog.arena_bytes <= kStaticArenaBytes) {
-      alt.c = c;
-      alt.swap();
-    }
+  if (outgrows_fixed_arena(c)) {
+    const ajf_status st = ajf_prepare_noalloc(c);  // enqueues nothing; no work when it was called before
+    if (st != AJF_OK) return st;
+    alt.c = c;
+    alt.swap();
   }
   const Program& P = c->prog;
-  if (P.arena_bytes > kStaticArenaBytes)
-    return fail(c, AJF_E_NOMEM, "plan needs " + std::to_string(P.arena_bytes) + " bytes of device memory; the fixed " +
-                                    "arena of ajf_fidelity_noalloc holds " + std::to_string(kStaticArenaBytes) + " bytes");
+  if (P.arena_bytes > kStaticArenaBytes) return fixed_arena_full(c, P.arena_bytes);
   if (!c->static_arena) return fail(c, AJF_E_STATE, "the fixed arena was not resolved when the context was created");
   CUDA_TRY(c, cudaSetDevice(c->device));
   // Run the same device program with the fixed arena as its base; the context's own arena, its

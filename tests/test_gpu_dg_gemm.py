@@ -1,5 +1,7 @@
 """The fp16 digit products that carry the GEMM-class steps of the F64 and F32 modes, through the
 path's own gather and GEMM, against extended-precision products and the CUDA-core GEMMs."""
+import time
+
 import numpy as np
 import pytest
 
@@ -96,6 +98,50 @@ def test_fixed_arena_takes_plans_that_only_digits_outgrow():
         n = ajf.ajf_fidelity_noalloc(c.handle, 1)
         again = ajf.ajf_fidelity_alg1(c.handle)
     assert abs(n["F"] - r["F"]) <= 1e-12 and again == r
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,gates,noises,seed,own", [(14, 170, 8, 1, False), (14, 170, 8, 2, True)])
+def test_fixed_arena_calls_only_enqueue_once_prepared(n, gates, noises, seed, own):
+    """Plans that fit the fixed arena with CUDA-core GEMMs only, on their own path (ajf_plan has lowered
+    it) and on one planned for it (ajf_prepare_noalloc): no call plans, which takes 0.6 s here against
+    milliseconds for the evaluation, and all agree."""
+    inst = W.mid(seed, n=n, n_gates=gates, n_noises=noises)
+    with ajf.Context(0) as c:
+        ajf.load_instance(c.handle, W.tiny(0))  # loads the kernels of the path
+        ajf.ajf_plan(c.handle, 2, trials=2)
+        ajf.ajf_fidelity_noalloc(c.handle, 2)
+        ajf.load_instance(c.handle, inst)
+        info = ajf.ajf_plan(c.handle, 2, trials=8)
+        assert info["arena_bytes"] > 64 << 20 and info["plan_seconds"] > 0.1
+        r = ajf.ajf_fidelity_alg2(c.handle)
+        if own:
+            ajf.ajf_prepare_noalloc(c.handle)
+        t = []
+        for _ in range(3):
+            t0 = time.perf_counter()
+            got = ajf.ajf_fidelity_noalloc(c.handle, 2)
+            t.append(time.perf_counter() - t0)
+            assert abs(got["F"] - r["F"]) <= 1e-12
+        assert t[0] < 3 * min(t) + 0.05
+        ajf.ajf_prepare_noalloc(c.handle)  # nothing left to do
+        ajf.load_instance(c.handle, W.mid(0))
+        ajf.ajf_plan(c.handle, 2, trials=2)
+        for call in (lambda: ajf.ajf_prepare_noalloc(c.handle), lambda: ajf.ajf_fidelity_noalloc(c.handle, 2)):
+            with pytest.raises(ajf.AjfError) as e:
+                call()
+            assert e.value.status == ajf.AJF_E_NOMEM
+
+
+def test_prepare_noalloc_needs_a_plan_and_a_device():
+    with ajf.Context(-1) as c:
+        ajf.load_instance(c.handle, W.tiny(0))
+        for plan in (False, True):
+            if plan:
+                ajf.ajf_plan(c.handle, 2, trials=2)
+            with pytest.raises(ajf.AjfError) as e:
+                ajf.ajf_prepare_noalloc(c.handle)
+            assert e.value.status == ajf.AJF_E_STATE
 
 
 @pytest.mark.parametrize("precision", ["f64", "f32"])
