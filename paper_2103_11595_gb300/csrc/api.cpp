@@ -2694,7 +2694,8 @@ ajf_status queue_table(ajf_ctx* const* ctxs, int n, double* dev_results, const Q
       switch (ln.kind) {
         case LK_SMALL:
           ph.kind = QK_SMALL;
-          ph.nblocks = ln.blocks;
+          ph.n = ln.blocks;
+          ph.nblocks = (ln.blocks + kQSmallGroups - 1) / kQSmallGroups;
           ph.count = ln.count;
           ph.desc = steps + ln.first;
           add(ph, -1);

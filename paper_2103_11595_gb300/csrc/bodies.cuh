@@ -36,11 +36,20 @@ namespace ajf {
 constexpr int kBodyThreads = 256;
 
 // Barrier policies of the bodies.
-struct SyncBlock {  // a standalone kernel of kBodyThreads threads
+struct SyncBlock {  // all threads of a standalone kernel
+  __device__ __forceinline__ static int tid() { return threadIdx.x; }
   __device__ __forceinline__ static void sync() { __syncthreads(); }
 };
 struct SyncBody {  // threads 0..kBodyThreads-1 of a larger block: named barrier 1
+  __device__ __forceinline__ static int tid() { return threadIdx.x; }
   __device__ __forceinline__ static void sync() { asm volatile("bar.sync 1, %0;" ::"n"(kBodyThreads) : "memory"); }
+};
+struct SyncSmall {  // one of the groups of kSmallThreads among those threads: named barriers 2, 3
+  __device__ __forceinline__ static int group() { return threadIdx.x / kSmallThreads; }
+  __device__ __forceinline__ static int tid() { return threadIdx.x % kSmallThreads; }
+  __device__ __forceinline__ static void sync() {
+    asm volatile("bar.sync %0, %1;" ::"r"(2 + group()), "n"(kSmallThreads) : "memory");
+  }
 };
 
 // Chained launches (kernels.h, launch_chained): the successor may start / everything before is complete.
@@ -87,14 +96,15 @@ __device__ __forceinline__ void build_table(const BitMap& m, int64_t* tab) {
 }
 // The tables of two maps over the same index (their instructions overlap).
 template <int kThreads = kBodyThreads>
-__device__ __forceinline__ void build_tables(const BitMap& m1, const BitMap& m2, int64_t* t1, int64_t* t2) {
+__device__ __forceinline__ void build_tables(const BitMap& m1, const BitMap& m2, int64_t* t1, int64_t* t2,
+                                             int tid = threadIdx.x) {
   const int nbits = m1.nbits, nc = nchunks(nbits);
   for (int c = 0; c < nc; ++c) {
     int64_t w1[8], w2[8];
     chunk_weights(m1, c, w1);
     chunk_weights(m2, c, w2);
     const int bits = nbits - 8 * c < 8 ? nbits - 8 * c : 8;
-    for (int v = threadIdx.x; v < (1 << bits); v += kThreads) {
+    for (int v = tid; v < (1 << bits); v += kThreads) {
       t1[(c << 8) | v] = chunk_offset(w1, v);
       t2[(c << 8) | v] = chunk_offset(w2, v);
     }
@@ -248,13 +258,12 @@ __device__ __forceinline__ double widen(float x) {
 template <typename T, typename Acc, typename Sync, int kThreads = kBodyThreads>
 __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, int nsteps, int total_blocks,
                                            T* arena, int vb, int64_t* tab, StepDev& st) {
-  const int s = find_step(steps, nsteps, vb);
+  const int s = find_step(steps, nsteps, vb), tid = Sync::tid();
   const int end = (s + 1 < nsteps) ? steps[s + 1].block0 : total_blocks;
   static_assert(sizeof(StepDev) % 4 == 0, "descriptor copy");
-  for (int i = threadIdx.x; i < static_cast<int>(sizeof(StepDev) / 4); i += kThreads)
+  for (int i = tid; i < static_cast<int>(sizeof(StepDev) / 4); i += kThreads)
     reinterpret_cast<int32_t*>(&st)[i] = reinterpret_cast<const int32_t*>(&steps[s])[i];
   Sync::sync();
-  if (int64_t(vb - st.block0) * kThreads >= int64_t(1) << st.rc) return;  // more blocks than outputs: all threads
   const int nb = end - st.block0;
   const int c_oa = nchunks(st.oa.nbits), c_ob = nchunks(st.ob.nbits);
   const int c_ka = nchunks(st.ka.nbits), c_kb = nchunks(st.kb.nbits);
@@ -262,8 +271,8 @@ __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, in
   int64_t* t_ob = t_oa + c_oa * 256;
   int64_t* t_ka = t_ob + c_ob * 256;
   int64_t* t_kb = t_ka + c_ka * 256;
-  build_tables<kThreads>(st.oa, st.ob, t_oa, t_ob);
-  build_tables<kThreads>(st.ka, st.kb, t_ka, t_kb);
+  build_tables<kThreads>(st.oa, st.ob, t_oa, t_ob, tid);
+  build_tables<kThreads>(st.ka, st.kb, t_ka, t_kb, tid);
   chain_wait();
   Sync::sync();
   const int64_t nout = int64_t(1) << st.rc, nk = int64_t(1) << st.rk;
@@ -275,7 +284,7 @@ __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, in
   with_operands(arena, st.a, st.fa, st.b, st.fb, [&](const auto* A, const auto* B) {
     using TA = typename std::remove_cv<typename std::remove_pointer<decltype(A)>::type>::type;
     using TB = typename std::remove_cv<typename std::remove_pointer<decltype(B)>::type>::type;
-    for (int64_t o = int64_t(vb - st.block0) * kThreads + threadIdx.x; o < nout; o += int64_t(nb) * kThreads) {
+    for (int64_t o = int64_t(vb - st.block0) * kThreads + tid; o < nout; o += int64_t(nb) * kThreads) {
       const auto* Ao = A + lookup(t_oa, c_oa, o);
       const auto* Bo = B + lookup(t_ob, c_ob, o);
       Acc re = 0, im = 0;

@@ -19,6 +19,8 @@ constexpr int kMaxBits = 48;
 // Threads of a small-step block (k_small). An SM adds FP64 products at 2 per clock, so a step of a few
 // hundred outputs is spread over as many SMs as its warps allow: 128 rather than 256 per block.
 constexpr int kSmallThreads = 128;
+// The interpreter's 256 body threads run this many of them side by side.
+constexpr int kQSmallGroups = 2;
 
 // Map from the bits of an index to element offsets of one tensor: offset(idx) =
 // sum_i bit_i(idx) << pos[i] (pos < 0: the bit does not address this tensor). Evaluated on the
@@ -162,7 +164,8 @@ struct QPhase {
   int32_t bn;          // QK_GEMM: tile width
   int32_t ksplit;      // QK_SPLIT_SUM: splits
   int32_t pad;
-  int64_t n;           // QK_SPLIT_SUM: elements of the result
+  int64_t n;           // QK_SPLIT_SUM: elements of the result; QK_SMALL: blocks of the launch, nblocks
+                       // of kQSmallGroups each
   char* base;          // the program's arena
   const void* desc;    // steps / perms / leaves / final record (device)
   const void* gemm;    // QK_GEMM: the GEMM's parameter block (device, 64-byte aligned)

@@ -72,9 +72,15 @@ __device__ __noinline__ void q_leaves(const QPhase& ph, int v) {
   leaf_body<double>(static_cast<const LeafDev*>(ph.desc), ph.p0, reinterpret_cast<double*>(ph.base), v);
 }
 __device__ __noinline__ void q_small(const QPhase& ph, int v, uint8_t* smem) {
-  small_body<double, double, SyncBody>(static_cast<const StepDev*>(ph.desc), ph.count, ph.nblocks,
-                                       reinterpret_cast<double*>(ph.base), v, reinterpret_cast<int64_t*>(smem),
-                                       *reinterpret_cast<StepDev*>(smem + kQArrays));
+  // a launch's blocks have 128 threads: two of them at a time, each with its own tables and descriptor
+  // (one at a time with 256 threads left half of those without an output)
+  static_assert(kQSmallGroups * kSmallThreads == kBodyThreads, "groups of the body threads");
+  static_assert(4 * ((kMaxBits + 7) / 8) * 256 * sizeof(int64_t) <= kQArrays / kQSmallGroups, "room for any step's tables");
+  const int g = SyncSmall::group(), vb = kQSmallGroups * v + g;
+  if (vb >= ph.n) return;
+  small_body<double, double, SyncSmall, kSmallThreads>(
+      static_cast<const StepDev*>(ph.desc), ph.count, static_cast<int>(ph.n), reinterpret_cast<double*>(ph.base), vb,
+      reinterpret_cast<int64_t*>(smem + g * (kQArrays / kQSmallGroups)), reinterpret_cast<StepDev*>(smem + kQArrays)[g]);
 }
 __device__ __noinline__ void q_splitk(const QPhase& ph, int v, uint8_t* smem) {
   double* red = reinterpret_cast<double*>(smem + kQArrays);
