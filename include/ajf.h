@@ -64,10 +64,9 @@ enum {
 };
 
 enum {
-  AJF_PREC_F64 = 0,    /* FP64 accuracy everywhere (GEMM-class steps: exact fp16 digit products
-                          on tcgen05, 64-bit fixed-point sums; FP64 CUDA cores without tcgen05) */
-  AJF_PREC_F32 = 1,    /* GEMM-class steps at FP32 accuracy (the same with fewer digits; FP32
-                          CUDA cores without tcgen05)                                          */
+  AJF_PREC_F64 = 0,    /* FP64 arithmetic; GEMM-class steps on tcgen05 to FP64 accuracy normwise
+                          per operand row (see below)                                          */
+  AJF_PREC_F32 = 1,    /* the same with GEMM-class steps to FP32 accuracy normwise per operand row */
   AJF_PREC_TF32 = 2,   /* GEMM-class steps: one-pass TF32 tensor-core GEMMs (tcgen05), FP32 accumulate */
   AJF_PREC_TF32X3 = 3, /* split TF32 hi/lo operands, three tcgen05 products, FP32 accumulate   */
   AJF_PREC_BF16X3 = 4, /* bf16 operands split in two terms, three tcgen05 products             */
@@ -79,7 +78,15 @@ enum {
  * the reduced modes' GEMM-class steps, which are complex64 (FP32 planes; each value is one FP32
  * register sum of the GEMM, so nothing is lost). A mode sets how the operands of the GEMM-class
  * steps are rounded or split. Leaves, small steps, the final contraction to a scalar,
- * sum_i |t_i|^2, F_J and 1 - F_J are FP64 in every mode. */
+ * sum_i |t_i|^2, F_J and 1 - F_J are FP64 in every mode.
+ *
+ * The GEMM-class steps of the F64 and F32 modes are exact products of fixed-point fp16 digits, summed
+ * in 64-bit fixed point and rounded once (FP64 or FP32 on CUDA cores where there is no tcgen05 or the
+ * memory budget has no room for the digits). An operand entry is kept to 2^-56 (F64) or 2^-38 (F32) of
+ * its row's largest entry, so the error of a product is bounded by the row norms |x_i| |y_j|, as F_J's
+ * is by the tensors' norms; it is not bounded by the sum of |x_ik| |y_jk|, as that of an FP64 or FP32
+ * sum is. Entries far below their row's largest keep fewer bits than FP64's 53 (FP32's 24) and, below
+ * 2^-63 of it, none. An open Kraus index of Alg. I is a row index: traces of small weight keep theirs. */
 
 enum {
   AJF_LOWER_DEFAULT = 0,   /* GEMM-class steps on tensor cores / CUDA-core GEMMs, one launch per

@@ -9,8 +9,13 @@
 // (|X| <= 2^62; exact for entries within 2^-9 of m) and written in balanced base 512:
 //   X = sum_{t < T} d_t 2^(54 - 9 t) + rest,   d_0 in [-256, 256], d_t in [-256, 255] (t >= 1).
 // Every digit is an integer that fp16 holds exactly. The last digit also takes the rest, rounded
-// to fp16's 11 significant bits. T = 6 keeps x to 2^-57 m (FP64 operands), T = 4 to 2^-39 m
-// (operands of the FP32 mode).
+// to fp16's 11 significant bits. T = 6 keeps x to 2^-56 m (FP64 operands), T = 4 to 2^-38 m
+// (operands of the FP32 mode): normwise per row, an entry below m in the fewer bits the smaller it is. On
+// rows graded over 10^6 the error over sum |a||b| is 1.6e-14 (FP64 sums: 4e-16), and 4.4e-12 where the two
+// operands are graded oppositely along the sum (tests/test_gpu_dg_gemm.py). The networks contracted here
+// do not show it: n = 8 .. 16 circuits with noises of 1e-2 down to 1e-12 (346 GEMMs) gave the same largest
+// |dF| as FP64 sums, 4.2e-15, and every one of 4096 traces to 3.2e-15 of its own Kraus weight, since an
+// open Kraus index is a row index; FP32: 5.7e-9 against 2.1e-8 on CUDA cores.
 //
 // Layout of a digit operand of R rows (a power of two >= 16) and Kr = 2K real columns (a power of
 // two >= 16): [row block of RB = min(R, 128)][chunk of 64 columns][slot][RB rows x 128 bytes], each

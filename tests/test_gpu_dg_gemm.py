@@ -211,3 +211,63 @@ def test_auto_slicing_leaves_plans_whole_that_fit_with_either_gemm(precision):
         assert auto["n_sliced_bonds"] == 0 and auto["arena_bytes"] == plain["arena_bytes"] <= budget
     tight = plan(smallest - 1, slice_bonds="auto")
     assert tight["n_sliced_bonds"] == 1 and tight["n_tc_gemms"] > 0 and tight["arena_bytes"] < smallest
+
+
+def row_bound(A, B, R, f32):
+    """Error bound of a digit product against row maxima m (per factor, real parts and imaginary ones), term
+    by term. Operands: the last digit's rounding, 2^-56 m (2^-38 m with four digits), on either side.
+    Dropped levels, 2^-14 q^2 = m^2 units of 2^(-9 l): 4 pairs of digits at l = 7, 3 at l = 4, and less than
+    1% below. Tensor-core sums (64 columns, at most 2^16 per product, 16 products and the running sum to an
+    addition, each truncated to a unit of the sum): with six digits exact up to 2^24, so one unit of 2 for
+    each of 4 x 17 terms at level 4, where the sum can pass it; with four digits, where the last one has a
+    fraction, one unit for each of 16 x 17 terms at level 3. Fixed point: three roundings per chunk in
+    units of 2^-54 (chunks per sum). The result's own rounding."""
+    K2 = 2 * A.shape[1]
+    m = np.maximum(abs(A.real), abs(A.imag)).max(1)[:, None] * np.maximum(abs(B.real), abs(B.imag)).max(1)[None, :]
+    chunks = max(1, K2 // 64)
+    per = K2 * (2 * 2.0 ** -38 + 3.03 * 2.0 ** -34 if f32 else 2 * 2.0 ** -56 + 4.04 * 2.0 ** -61)
+    per += chunks * (272 * 2.0 ** -41 if f32 else 136 * 2.0 ** -50) + 1.5 * chunks * min(chunks, 32) * 2.0 ** -54
+    return 2.0 ** (-24 if f32 else -53) * 1.01 * np.maximum(abs(R[0]), abs(R[1])).astype(float) + m * per
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("K", [8, 16, 64, 4096])  # four, two and one digits per 128-byte row; K splits
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_digit_gemm_with_the_largest_digits(precision, K):
+    """Entries whose digits all are the largest that they can be (255 and -255; 256 and -256): the exact
+    levels' sums come within 1% of the 2^24 that FP32 holds, and the fixed-point sums to their largest."""
+    T = 4 if precision == "f32" else 6
+    places = [2.0 ** (-9 * t) for t in range(T)]
+    same = 255.0 * sum(places)                  # 255 in every place
+    mixed = 256.0 - 256.0 * sum(places[1:])     # 256, then -256
+    for a in (same, -same, mixed):
+        for b in (same, mixed):
+            for za, zb in ((1 - 1j, 1 + 1j), (1 + 1j, 1 + 1j)):  # all terms of Re, and of Im, of one sign
+                A, B = np.full((32, K), a * za), np.full((32, K), b * zb)
+                R = exact(A, B)
+                C = ajf.ajf_selftest_digit_gemm(0, precision, A, B)
+                err = np.maximum(abs(C.real - R[0]), abs(C.imag - R[1])).astype(float)
+                assert (err <= row_bound(A, B, R, precision == "f32")).all(), (a, b, err.max())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("decades", [3, 6, 10, 12])
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_digit_gemm_is_normwise_per_row(precision, decades):
+    """Entries graded within their rows, at random and oppositely in the two operands: the error is bounded
+    by the row maxima, not by sum |a||b| (the figure printed, with the CUDA-core GEMM's)."""
+    r = np.random.default_rng(decades)
+    M, N, K = 32, 32, 64
+    A = r.standard_normal((M, K)) + 1j * r.standard_normal((M, K))
+    B = r.standard_normal((N, K)) + 1j * r.standard_normal((N, K))
+    grade = 10.0 ** -np.linspace(0, decades, K)
+    for name, fa, fb in (("random", 10.0 ** r.uniform(-decades, 0, (M, K)), 10.0 ** r.uniform(-decades, 0, (N, K))),
+                         ("opposed", grade, grade[::-1])):
+        a, b = A * fa, B * fb
+        R = exact(a, b)
+        C = ajf.ajf_selftest_digit_gemm(0, precision, a, b)
+        S = ajf.ajf_selftest_digit_gemm(0, precision, a, b, digits=False)
+        e, es = (np.maximum(abs(X.real - R[0]), abs(X.imag - R[1])).astype(float) for X in (C, S))
+        mag = abs(a) @ abs(b).T
+        print(f"{precision} {name} 10^-{decades}: error / sum |a||b| {(e / mag).max():.1e} (CUDA cores {(es / mag).max():.1e})")
+        assert (e <= row_bound(a, b, R, precision == "f32")).all()
