@@ -52,13 +52,14 @@ struct SyncSmall {  // one of the groups of kSmallThreads among those threads: n
   }
 };
 
-// Chained launches (kernels.h, launch_chained): the successor may start / everything before is complete.
+// Chained launches (kernels.h, launch_chained): everything before is complete, and (early) the successor
+// may start. In this order: at most two kernels of a chain overlap.
 // The bodies below run in such kernels, and as tasks of the interpreter beside the blocks that write their
 // operands: their pointers to tensors and partial sums are not __restrict__.
-__device__ __forceinline__ void chain_trigger(bool early) {
+__device__ __forceinline__ void chain_wait(bool early = false) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ------------------------------------------------------------------ offset tables
 
@@ -257,7 +258,7 @@ __device__ __forceinline__ double widen(float x) {
 // clocks.
 template <typename T, typename Acc, typename Sync, int kThreads = kBodyThreads>
 __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, int nsteps, int total_blocks,
-                                           T* arena, int vb, int64_t* tab, StepDev& st) {
+                                           T* arena, int vb, int64_t* tab, StepDev& st, bool early = false) {
   const int s = find_step(steps, nsteps, vb), tid = Sync::tid();
   const int end = (s + 1 < nsteps) ? steps[s + 1].block0 : total_blocks;
   static_assert(sizeof(StepDev) % 4 == 0, "descriptor copy");
@@ -273,7 +274,7 @@ __device__ __forceinline__ void small_body(const StepDev* __restrict__ steps, in
   int64_t* t_kb = t_ka + c_ka * 256;
   build_tables<kThreads>(st.oa, st.ob, t_oa, t_ob, tid);
   build_tables<kThreads>(st.ka, st.kb, t_ka, t_kb, tid);
-  chain_wait();
+  chain_wait(early);
   Sync::sync();
   const int64_t nout = int64_t(1) << st.rc, nk = int64_t(1) << st.rk;
   const bool one_chunk = c_ka == 1;  // (no chunk, rk = 0: lookup gives 0)
@@ -1016,7 +1017,7 @@ __device__ __forceinline__ void perm_tiles_bf16x3(const PermDev& p, const double
 template <typename S, typename Sync>
 __device__ __forceinline__ void perm_body(const PermDev* __restrict__ perms, const double* arena,
                                           char* base, int vb, int vg, int vy, int64_t* tab,
-                                          PermSmem<S>& sm, PermSmem<float>* sm2 = nullptr) {
+                                          PermSmem<S>& sm, PermSmem<float>* sm2 = nullptr, bool early = false) {
   constexpr int TKMAX = PermSmem<S>::TKMAX;
   auto& tre = sm.tre;
   auto& tim = sm.tim;
@@ -1030,7 +1031,7 @@ __device__ __forceinline__ void perm_body(const PermDev* __restrict__ perms, con
   int64_t* t_k = tab + c_r * 256;
   build_table(p.rows, t_r);
   build_table(p.cols, t_k);
-  chain_wait();
+  chain_wait(early);
   Sync::sync();
   if constexpr (sizeof(S) == 4) {
     if (p.mode == OPM_BF16X3 && p.rbits >= 5 && p.kbits >= 6) {

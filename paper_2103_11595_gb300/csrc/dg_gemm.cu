@@ -214,7 +214,7 @@ __device__ __forceinline__ uint4 neg_f16x8(uint4 v) {
 // planes in one thread a block's chain of some 1,000 instructions per tile took 24 us even alone.
 template <typename S, int T>
 __device__ __forceinline__ void digits_body(const PermDev& p, const S* src, char* base,
-                                            int64_t* tab, S* tre, S* tim) {
+                                            int64_t* tab, S* tre, S* tim, bool early) {
   const int c_r = nchunks(p.rows.nbits), c_k = nchunks(p.cols.nbits);
   int64_t* t_r = tab;
   int64_t* t_k = tab + c_r * 256;
@@ -235,7 +235,7 @@ __device__ __forceinline__ void digits_body(const PermDev& p, const S* src, char
   const bool unit = u < (1 << (p.tr + p.tk - 3));
   const int urow = (u << 3) >> p.tk, uk = (u << 3) & ((1 << p.tk) - 1);
   const int lanes = 1 << (p.tk - 3);               // units of one row of the tile
-  chain_wait();
+  chain_wait(early);
   __syncthreads();
   const unsigned units = __ballot_sync(0xffffffffu, unit);  // lanes that take part in a row's reduction
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -313,15 +313,14 @@ template <int T>
 __global__ void __launch_bounds__(kDigThreads, 2) k_digits(const PermDev* __restrict__ perms,
                                                            const double* arena, char* base,
                                                            bool early) {
-  chain_trigger(early);
   extern __shared__ int64_t tab[];
   __shared__ __align__(16) double tile[2 * kTileElems];
   const PermDev& p = perms[blockIdx.y];
   if (p.src_f32) {
     float* t = reinterpret_cast<float*>(tile);
-    digits_body<float, T>(p, reinterpret_cast<const float*>(arena) + p.src, base, tab, t, t + kTileElems);
+    digits_body<float, T>(p, reinterpret_cast<const float*>(arena) + p.src, base, tab, t, t + kTileElems, early);
   } else {
-    digits_body<double, T>(p, arena + p.src, base, tab, tile, tile + kTileElems);
+    digits_body<double, T>(p, arena + p.src, base, tab, tile, tile + kTileElems, early);
   }
 }
 
@@ -409,7 +408,6 @@ __device__ __forceinline__ void mad_high(int64_t& acc, int v, int mul) { acc += 
 
 template <int BC, int T, int PACK, typename Out>
 __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__ DgParams p) {
-  chain_trigger(p.early != 0);
   constexpr int kLevels = T == 6 ? 7 : 4;
   constexpr int COLS = BC / 4;                 // columns per epilogue thread
   constexpr int CH = COLS < 16 ? COLS : 16;    // columns per TMEM load
@@ -446,7 +444,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dg_gemm(const __grid_constant__
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = __shfl_sync(0xffffffffu, *sh.tmem_slot, 0);
-  chain_wait();
+  chain_wait(p.early != 0);
 
   // work item wi: tile wi % tiles of K split wi / tiles; `group` Y blocks sweep the X blocks together
   const uint32_t tiles = static_cast<uint32_t>(p.nty) * static_cast<uint32_t>(p.ntx);

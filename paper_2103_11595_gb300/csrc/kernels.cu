@@ -39,8 +39,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(const StepDev* __restri
                                                          int total_blocks, T* arena, bool early) {
   extern __shared__ int64_t tab[];
   __shared__ StepDev st;
-  chain_trigger(early);
-  small_body<T, Acc, SyncBlock, kSmallThreads>(steps, nsteps, total_blocks, arena, blockIdx.x, tab, st);
+  small_body<T, Acc, SyncBlock, kSmallThreads>(steps, nsteps, total_blocks, arena, blockIdx.x, tab, st, early);
 }
 
 template <typename T>
@@ -80,12 +79,11 @@ __global__ void __launch_bounds__(kBodyThreads, 4) k_perm(const PermDev* __restr
                                                        bool early) {
   extern __shared__ int64_t tab[];
   __shared__ PermSmem<S> sm;
-  chain_trigger(early);
   if constexpr (sizeof(S) == 4) {
     __shared__ PermSmem<float> sm2;  // second tile buffer of the six-product split's copy pipeline
-    perm_body<S, SyncBlock>(perms, arena, base, blockIdx.x, gridDim.x, blockIdx.y, tab, sm, &sm2);
+    perm_body<S, SyncBlock>(perms, arena, base, blockIdx.x, gridDim.x, blockIdx.y, tab, sm, &sm2, early);
   } else {
-    perm_body<S, SyncBlock>(perms, arena, base, blockIdx.x, gridDim.x, blockIdx.y, tab, sm);
+    perm_body<S, SyncBlock>(perms, arena, base, blockIdx.x, gridDim.x, blockIdx.y, tab, sm, nullptr, early);
   }
 }
 

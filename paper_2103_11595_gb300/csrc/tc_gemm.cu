@@ -69,7 +69,6 @@ using namespace tc;
 
 template <int BN, int kKind, int kT>
 __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__ TcParams p, bool early) {
-  chain_trigger(early);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5;
@@ -88,7 +87,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   sh.tmem = *tmem_slot;
-  chain_wait();
+  chain_wait(early);
   TcRing ring;
   const uint32_t nwork = static_cast<uint32_t>(p.tiles) * static_cast<uint32_t>(p.ksplit);
   tc_gemm_terms<BN, kKind, kT>(p, blockIdx.x, nwork, gridDim.x, sh, ring);

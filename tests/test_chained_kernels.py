@@ -35,6 +35,17 @@ def test_chained_kernels_promise_nothing_about_others_data(name):
         assert set(restrict_params(text, k)) <= DESCRIPTORS, k
 
 
+def test_a_kernel_lets_its_successor_start_after_its_own_wait():
+    """So that at most two kernels of a chain are resident: the trigger is only ever issued behind the wait."""
+    found = 0
+    for name in sorted(os.listdir(CSRC)):
+        text = source(name)
+        for m in re.finditer(r"griddepcontrol\.launch_dependents", text):
+            found += 1
+            assert "griddepcontrol.wait" in text[:m.start()].rsplit("{", 1)[1], name
+    assert found == 1
+
+
 def test_shared_bodies_promise_nothing_about_others_data():
     for name in ("bodies.cuh", "dg_gemm.cu"):
         text = source(name)
@@ -80,6 +91,21 @@ def test_repeated_scaled_fp16_evaluations_are_bitwise_equal(seed):
             ajf.ajf_plan(c.handle, 2, precision="f16x3", trials=8, use_graph=k % 2 == 1)
             seen |= {ajf.ajf_fidelity_alg2(c.handle)["S"] for _ in range(25)}
     assert len(seen) == 1
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", ["f64", "f32", "bf16x6", "tf32x3", "f16x3"])
+def test_first_evaluations_are_bitwise_equal(precision):
+    """New contexts, one evaluation each, the launches enqueued one by one."""
+    for seed in (0, 3):
+        inst = W.mid(seed)
+        seen = set()
+        for _ in range(25):
+            with ajf.Context(0) as c:
+                ajf.load_instance(c.handle, inst)
+                ajf.ajf_plan(c.handle, 2, precision=precision, trials=8)
+                seen.add(ajf.ajf_fidelity_alg2(c.handle)["S"])
+        assert len(seen) == 1
 
 
 @pytest.mark.gpu
