@@ -504,6 +504,12 @@ __device__ __forceinline__ bool tc_gemm_terms(const TcParams& p, uint32_t wi0, u
             for (int j = 0; j < CH; ++j) acc[c0 + j] += __uint_as_float(r0[j]);
           }
         }
+        // Scaled fp16: the arrival also gives buffer b's scales back, which the issuer then overwrites with a
+        // bulk copy (async proxy). The reads above are generic ones, and neither __syncwarp nor the arrival
+        // orders them before writes of the other proxy: without the fence a warp's last scales could
+        // come from the K block that uses the buffer next (about one n = 16 evaluation in 5,000 off by up
+        // to 3e-5, in blocks of the last four columns read).
+        if (kKind == 2) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(sh.acce0 + 8 * b);

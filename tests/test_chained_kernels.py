@@ -61,6 +61,14 @@ def test_epilogue_lanes_wait_for_what_they_read():
     assert "if (lane == 0) w" not in epilogue and "__shfl_sync" not in epilogue
 
 
+def test_scales_are_given_back_across_the_proxies():
+    """The scaled fp16 epilogue reads its scales through the generic proxy, and the issuer overwrites them
+    with a bulk copy once the buffer's barrier has been arrived at: a proxy fence stands between."""
+    epilogue = source("tc_gemm_dev.cuh").split("} else if (warp >= kEpiWarp0) {")[1].split("mbar_arrive(sh.acce0")[0]
+    last_read = epilogue.rindex("(sbv + c0 + j)")
+    assert "if (kKind == 2) asm volatile(\"fence.proxy.async.shared::cta;\"" in epilogue[last_read:]
+
+
 def test_warp_operations_name_their_lanes():
     """A shuffle or vote over whichever lanes happen to be together drops the others' values: the masks
     come from the conditions that the lanes are under."""
