@@ -3,10 +3,11 @@
 // persistent step interpreter (queue.cu: one launch for many programs, whose thread blocks run
 // these bodies as tasks with virtual block indices).
 //
-// Every body runs on kBodyThreads = 256 threads (threads 0..255 of the block) and synchronises
-// them through the Sync policy: __syncthreads() in a standalone kernel, a named barrier of those
-// 256 threads in the interpreter, whose blocks carry more warps. Shared-memory scratch comes in
-// through pointers, so that the interpreter can place it in its own dynamic shared memory.
+// A body runs on kBodyThreads = 256 threads (threads 0..255 of the block), small_body on
+// kSmallThreads = 128, and synchronises them through the Sync policy: __syncthreads() in a standalone
+// kernel, a named barrier of those threads in the interpreter, whose blocks carry more warps and run two
+// small bodies side by side. Shared-memory scratch comes in through pointers, so that the interpreter can
+// place it in its own dynamic shared memory.
 //
 //  leaf_body        builds a leaf tensor of the miter network from the uploaded complex128
 //                   gate/Kraus matrices (gate, conjugate, adjoint, transpose, Kraus stack with an
@@ -19,7 +20,7 @@
 //  perm_body        gathers a complex tensor into a real, K-contiguous GEMM operand (the complex
 //                   product C = A B becomes the real product [[Ar,-Ai],[Ai,Ar]] [Br;Bi] = [Cr;Ci]),
 //                   in the operand format of the precision mode.
-//  split_sum_body   sums the FP64 K-split partial tiles of a tensor-core GEMM in a fixed order.
+//  split_sum_body   sums the FP32 K-split partial tiles of a tensor-core GEMM in a fixed order.
 //  open_body/final_body  the FP64 end of the path: t_i for Alg. I, sum |t_i|^2, F_J and 1 - F_J.
 #pragma once
 #include <cuda_bf16.h>

@@ -13,14 +13,16 @@
 // i + j = l share the weight q_x q_y 2^(-9 l): level l is one tensor-core accumulation of l + 1
 // digit products over a chunk of 64 columns. Its value is an integer of at most
 // (l + 1) 2^16 64 <= 2^24 for l <= 3, so the tensor core's FP32 accumulation (which truncates) is
-// exact there; levels 4 and up are below 2^-36 of the leading level's range, where its truncation
-// is below 2^-58 of q_x q_y 2^14. The epilogue converts every level to an integer and adds it, shifted, into a
-// 64-bit fixed-point register sum (unit q_x q_y 2^-sh0), which is rounded once, to FP64, at the
-// end. An FP64 CUDA-core product rounds at every one of its K additions; both errors against exact
+// exact there -- but for the last digit, which carries the rest: with four digits level 3 is truncated to
+// 2^-27 q_x q_y, 2^-41 of the row maxima's product. Levels 4 and up can pass 2^24 when nearly all digits
+// are at their largest and of one sign; a truncation is then 2^-35 q_x q_y, 2^-49 of that product. The epilogue
+// converts every level to an integer and adds it, shifted, into a 64-bit fixed-point register sum (unit
+// q_x q_y 2^-sh0), which is rounded once, to FP64, at the end. An FP64 CUDA-core product rounds at every one of its K additions; both errors against exact
 // products are compared in tests/test_gpu_dg_gemm.py. FP64 keeps 7 levels (26 digit products) at
 // every K: without the seventh (about 2^-54 of the row maxima's product per column) the error was
 // 1.5 to 2 times a CUDA-core sum's on normally distributed operands at K = 1024 .. 8192, and up to 15
-// times on operands graded over 10^3; with it, 0.3 to 0.7 times. The FP32 mode keeps 4 (10 products).
+// times on operands graded over 10^3; with it, 0.3 to 0.7 times (in the norm; digits.cuh says what that leaves
+// open). The FP32 mode keeps 4 (10 products).
 //
 // k_dg_gemm, structure: persistent, one CTA per SM, 640 threads: bulk-copy producer warp, MMA issuer
 // warp, two idle warps, sixteen epilogue warps. The M = 128 side of the MMA is Y's rows (the larger

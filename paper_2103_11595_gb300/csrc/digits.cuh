@@ -13,7 +13,7 @@
 // (operands of the FP32 mode): normwise per row, an entry below m in the fewer bits the smaller it is. On
 // rows graded over 10^6 the error over sum |a||b| is 1.6e-14 (FP64 sums: 4e-16), and 4.4e-12 where the two
 // operands are graded oppositely along the sum (tests/test_gpu_dg_gemm.py). The networks contracted here
-// do not show it: n = 8 .. 16 circuits with noises of 1e-2 down to 1e-12 (346 GEMMs) gave the same largest
+// do not show it: n = 8 .. 16 circuits with noises of 1e-2 down to 1e-12 (692 GEMMs) gave the same largest
 // |dF| as FP64 sums, 4.2e-15, and every one of 4096 traces to 3.2e-15 of its own Kraus weight, since an
 // open Kraus index is a row index; FP32: 5.7e-9 against 2.1e-8 on CUDA cores.
 //
@@ -21,7 +21,8 @@
 // two >= 16): [row block of RB = min(R, 128)][chunk of 64 columns][slot][RB rows x 128 bytes], each
 // RB x 128-byte tile in the 128-byte swizzle that the MMA reads, so a tile is one contiguous bulk
 // copy. With Kr >= 64 slot t holds digit t. A narrower operand packs 2 (Kr = 32) or 4 (Kr = 16)
-// digits side by side in one 128-byte row, so that no bytes are spent on padding columns.
+// digits side by side in one 128-byte row, so that no bytes are spent on padding columns (with six digits
+// and four to a row, two of the eight places stay unused).
 #pragma once
 #include <cuda_runtime.h>
 

@@ -26,7 +26,8 @@
 namespace ajf {
 
 // ------------------------------------------------------------------ standalone kernels
-// (the bodies are in bodies.cuh; one launch per program step, 256 threads per block)
+// (the bodies are in bodies.cuh; one launch per level of small steps or per step, 256 threads per block, 128 in
+// k_small)
 
 template <typename T>
 __global__ void __launch_bounds__(kBodyThreads) k_leaf(const LeafDev* leaves, const double* __restrict__ in,

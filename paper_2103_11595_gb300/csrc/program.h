@@ -66,8 +66,8 @@ struct Program {
 
 // Lower `path` over `net` to a device program for `precision`. `inputs_complex` is the number
 // of complex128 values in the packed input buffer. `tc_ok`: tensor-core GEMMs may be used;
-// `digits`: also those of the F64 and F32 modes (digit operands, which take up to 1.5 times the
-// memory of the CUDA-core GEMMs' operands).
+// `digits`: also those of the F64 and F32 modes (digit operands, which take 1.5 to 2 times
+// the memory of the CUDA-core GEMMs' operands).
 // `persistent`: every step becomes a CUDA-core gather step (LK_SMALL) or a reduction step
 // (LK_SPLITK), so that one thread block of the persistent kernel can run the whole program.
 Program lower(const Network& net, const Path& path, int precision, size_t inputs_complex, bool tc_ok,

@@ -95,9 +95,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gemm_tc(const __grid_constant__
     tc_drain_after_abort(p.slots, p.bufs, p.wait_ns, p.status, sh, ring);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   // __syncthreads (bar.sync, the aligned form) must be executed by all threads of a warp
-  // together; warps 0 and 1 get here diverged (lane 0 ran the producer / MMA loop, lanes 1-31 came
-  // straight through), so they reconverge first. The barrier then orders warp 1's TMEM release
-  // after every epilogue warp's last TMEM read and after the abort drains above.
+  // together, so a warp whose lanes left the roles or the drain apart reconverges first. The barrier then
+  // orders warp 1's TMEM release after every epilogue warp's last TMEM read and after the abort drains above.
   __syncwarp();
   __syncthreads();
   if (warp == 1) {
