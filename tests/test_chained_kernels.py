@@ -53,12 +53,15 @@ def test_shared_bodies_promise_nothing_about_others_data():
             assert set(restrict_params(text, body)) <= DESCRIPTORS, body
 
 
-def test_epilogue_lanes_wait_for_what_they_read():
-    """No lane of the GEMM's epilogue reads scales or accumulators on another lane's word (a shuffle
-    orders no memory)."""
+def test_epilogue_lanes_read_behind_a_warp_barrier():
+    """No lane of the GEMM's epilogue reads scales or accumulators on another lane's word alone (a shuffle
+    orders no memory): a warp barrier stands behind each wait."""
     epilogue = source("tc_gemm_dev.cuh").split("} else if (warp >= kEpiWarp0) {")[1].split("if (mine) {")[0]
-    assert epilogue.count("mbar_wait(") == 2
-    assert "if (lane == 0) w" not in epilogue and "__shfl_sync" not in epilogue
+    waits = epilogue.split("mbar_wait(")[1:]
+    assert len(waits) == 2
+    for w in waits:
+        w = w[:w.index("if (!ok) break;")]
+        assert "__syncwarp();" in w[w.index("__shfl_sync("):]
 
 
 def test_scales_are_given_back_across_the_proxies():
