@@ -385,8 +385,8 @@ ajf_status ajf_fidelity_alg2(ajf_ctx *ctx, double eps, ajf_result *out);
  * __device__ array: every GPU that loads the library holds those 64 MiB until the process exits.
  * Plans of the F64 and F32 modes whose arena (ajf_workspace_size) exceeds 64 MiB run a program with
  * CUDA-core GEMMs instead, which needs less memory: it computes the same F_J and traces, rounded
- * differently, and slower. ajf_plan lowers it on the plan's own path; where it only fits on a path
- * planned for it, ajf_prepare_noalloc plans that path.
+ * differently, and slower. ajf_prepare_noalloc makes it: on the plan's own path, or where it only fits
+ * on a path planned for it, on that.
  * It calls no cudaMalloc, cudaFree, cudaMallocHost or other allocating routine; inputs are copied
  * from the context's host memory and the result is read back synchronously. The context's own
  * arena, CUDA graph and Alg. I trace buffer are not touched (ajf_alg1_traces still returns the
@@ -406,9 +406,10 @@ ajf_status ajf_fidelity_alg2(ajf_ctx *ctx, double eps, ajf_result *out);
 ajf_status ajf_fidelity_noalloc(ajf_ctx *ctx, int alg, double eps, ajf_result *out);
 
 /* Host-side preparation of ajf_fidelity_noalloc for the current plan (no device work): after it that
- * call only enqueues. It plans (as long as ajf_plan takes) for an F64 or F32 plan that fits the fixed
- * arena only with CUDA-core GEMMs on a path of their own, and returns at once for every other plan.
- * ajf_fidelity_noalloc prepares itself where this call was left out.
+ * call only enqueues. For an F64 or F32 plan that fits the fixed arena only with CUDA-core GEMMs it lowers
+ * that program (about 1 ms) and, where only a path of its own fits, plans it (as long as ajf_plan takes);
+ * for every other plan it returns at once. ajf_fidelity_noalloc prepares itself where this call was left
+ * out, once per plan.
  * Errors: AJF_E_ARG (NULL), AJF_E_STATE (no plan, host-only context, sliced plan), AJF_E_NOMEM (the
  * plan does not fit the fixed arena: ajf_fidelity_noalloc would fail the same way). */
 ajf_status ajf_prepare_noalloc(ajf_ctx *ctx);

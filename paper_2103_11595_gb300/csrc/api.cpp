@@ -1072,10 +1072,11 @@ bool outgrows_fixed_arena(const ajf_ctx* c) {
          c->opts.lowering != AJF_LOWER_PERSISTENT && !multi_run(c) && c->prog.arena_bytes > kStaticArenaBytes;
 }
 
-// That program: CUDA-core GEMMs on the plan's own path (made by ajf_plan: under 2 ms) or, with `search`, on
-// one planned for them if that one alone fits (as long as planning takes). Kept until the next plan;
-// alt_prog.arena_bytes is the smallest found.
-void prepare_fixed_arena(ajf_ctx* c, bool search) {
+// That program: CUDA-core GEMMs on the plan's own path (0.6 ms at n = 16) or, if that does not fit, on one
+// planned for them (as long as planning takes). Kept until the next plan; alt_prog.arena_bytes is the
+// smallest found. Not made by ajf_plan, which most callers follow with other evaluations (n = 16, structure
+// known: load and plan 2.2 -> 2.8 ms).
+void prepare_fixed_arena(ajf_ctx* c) {
   auto lower_plain = [&](const Path& path) {
     return lower(c->net, path, c->opts.precision, c->in.packed.size() / 2, c->tc_device, false, false);
   };
@@ -1086,7 +1087,7 @@ void prepare_fixed_arena(ajf_ctx* c, bool search) {
     c->alt_searched = false;
     c->alt_gen = c->prog_gen;
   }
-  if (!search || c->alt_searched || c->alt_prog.arena_bytes <= kStaticArenaBytes) return;
+  if (c->alt_searched || c->alt_prog.arena_bytes <= kStaticArenaBytes) return;
   PlanParams pp = plan_params(c->opts, false);
   std::vector<int64_t> key = cuda_core_key(c->plan_key);
   if (pp.planner == AJF_PLANNER_LEARNED) pp.planner = AJF_PLANNER_AUTO;
@@ -1412,12 +1413,6 @@ ajf_status plan_one(ajf_ctx* c, int alg, const ajf_plan_opts* opts, ajf_plan_inf
   for (int j : slice_noises) c->slice_leaves.push_back(c->net.noise_leaf[j]);
   c->planned = true;
   c->plan_gen++;
-  if (outgrows_fixed_arena(c)) {
-    try {
-      prepare_fixed_arena(c, false);
-    } catch (const std::exception&) {  // ajf_prepare_noalloc tries again, and reports
-    }
-  }
   c->err.clear();
   return AJF_OK;
 }
@@ -1758,7 +1753,7 @@ ajf_status ajf_prepare_noalloc(ajf_ctx* c) {
   size_t bytes = c->prog.arena_bytes;
   if (outgrows_fixed_arena(c)) {
     try {
-      prepare_fixed_arena(c, true);
+      prepare_fixed_arena(c);
     } catch (const std::exception& ex) {
       return fail(c, AJF_E_NOMEM, std::string("planning for the fixed arena failed: ") + ex.what());
     }

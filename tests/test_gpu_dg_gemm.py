@@ -103,9 +103,9 @@ def test_fixed_arena_takes_plans_that_only_digits_outgrow():
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,gates,noises,seed,own", [(14, 170, 8, 1, False), (14, 170, 8, 2, True)])
 def test_fixed_arena_calls_only_enqueue_once_prepared(n, gates, noises, seed, own):
-    """Plans that fit the fixed arena with CUDA-core GEMMs only, on their own path (ajf_plan has lowered
-    it) and on one planned for it (ajf_prepare_noalloc): no call plans, which takes 0.6 s here against
-    milliseconds for the evaluation, and all agree."""
+    """Plans that fit the fixed arena with CUDA-core GEMMs only, on their own path (no preparation needed:
+    lowering takes a millisecond) and on one planned for it (ajf_prepare_noalloc): no call plans, which takes
+    0.6 s here against milliseconds for the evaluation, and all agree."""
     inst = W.mid(seed, n=n, n_gates=gates, n_noises=noises)
     with ajf.Context(0) as c:
         ajf.load_instance(c.handle, W.tiny(0))  # loads the kernels of the path
